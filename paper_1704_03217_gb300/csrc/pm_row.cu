@@ -8,25 +8,25 @@
 // update.  A persistent CTA (one per SM) has PR_PROD producer warps and
 // pr_cons consumer warps around a ring of tile buffers in shared memory, each
 // with a "full" and an "empty" mbarrier:
-//   - producer warp p stages the CTA's tiles p, p + PR_PROD, ...: it waits
-//     until the tile's buffer is empty, reads the tile's seeds (one lane per
-//     seed), drops the propagated candidates that cannot change the result,
-//     draws the first Philox block of every seed, places the target window at
-//     the per-component median of the current matches, and issues three 2D
+//   - producer warp p stages the CTA's tiles p, p + PR_PROD, ...: it reads the
+//     tile's seeds (one lane per seed), drops the propagated candidates that
+//     cannot change the result, draws the first Philox block of every seed,
+//     places the target window at the per-component median of the current
+//     matches, waits until the tile's buffer is empty and issues three 2D
 //     tensor copies: the reference region of all the tile's patches
 //     (split-byte words, a = 128 a_h + a_l), the target window (int16 words)
 //     and the window's sums |b|^2;
-//   - consumer warps take the tile's seeds from a shared counter, release the
-//     buffer when the counter runs out and move on to the next tile.
+//   - consumer warps take the tile's seeds from a shared counter (gray: in
+//     turn), release the buffer when they run out and move on to the next tile.
 // The descriptors carry a replicated border of BORD pixels in memory, so every
 // patch whose centre lies in the image is read without clamping and every
 // staged region is one tensor copy (coordinates outside the padded image read
 // as zero and are never used).
 //
-// Consumer layout: a warp scores one seed at a time, up to two candidates per
-// round.  Lane l owns the pixels k = l, l + 32, ... of the P x P patch in
-// raster order and holds their reference words in registers (3 words per
-// pixel for 6 channels, 1 for 2); a colour pixel of the target is one 16-byte
+// Consumer layout (six channels; gray: two seeds per warp, k_pm_g below): a
+// warp scores one seed at a time.  Lane l owns the pixels k = l, l + 32, ... of
+// the P x P patch in raster order and holds their reference words in
+// registers (3 words per pixel); a colour pixel of the target is one 16-byte
 // load.  Reference region and window share one row pitch, congruent to P
 // modulo 8 pixels, so pixel k of any patch lies in the 16-byte bank quad
 // k + const (mod 8): the 8 lanes of a quarter-warp never collide.  The cross
@@ -135,6 +135,21 @@ struct __align__(16) RowRec {       // one active seed of a staged tile
     unsigned long long cost, sa;    // current cost, sum |a|^2 of the reference patch
 };
 
+// One active seed of a staged tile, int16 search: 80 bytes in 16-byte units.
+struct __align__(16) RowSeed {
+    int s, pxy, roff, fl;           // seed index (-1: none); centre (x low 16, y high 16); word
+                                    // offset of its reference patch; flags (below)
+    unsigned long long cost, sa;    // current cost, sum |a|^2 of the reference patch
+    int cand[5][2];                 // displacement and window slot of the current match, of the
+                                    // two propagated ones and of the first two search candidates
+                                    // around the current match
+    int r[2];                       // random-search offsets k = 0, 1 (packed like u)
+};
+// RowSeed::fl: the seed's flag byte after the refresh, the byte as read << 8,
+// candidates to score (bits of cand[]) << 16, search count K << 21
+__device__ __forceinline__ int sd_pend(int fl) { return (fl >> 16) & 31; }
+__device__ __forceinline__ int sd_k(int fl) { return (fl >> 21) & 15; }
+
 struct RowHdr { int pair, dir, rx0, ry0, wx0, wy0, use_win, shr, shw, shs, pad0, pad1; };
 
 // The flattened tiles of one launch: slot k owns tiles [cum[k], cum[k + 1]);
@@ -179,10 +194,6 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_tx(unsigned bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
@@ -220,6 +231,32 @@ __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 
+// Evaluation counts of a CTA, per pair and direction: propagation and search,
+// cost refresh, and those read from global memory; in shared memory until the
+// CTA ends.  (A global atomic per warp and tile was up to 180000 a launch on a
+// few addresses at 16 pairs of 1024 x 436, which hold up every other access to
+// memory: 9.57 -> 9.43 ms a colour step.)
+struct EvCount { unsigned n[MAXB][2][3]; };
+__device__ __forceinline__ void ev_clear(EvCount& ev) {
+    for (int i = threadIdx.x; i < MAXB * 6; i += blockDim.x) (&ev.n[0][0][0])[i] = 0u;
+}
+__device__ __forceinline__ void ev_add(EvCount& ev, const RowHdr& H, unsigned n_eval,
+                                       unsigned n_cost, unsigned n_glob) {
+    unsigned* c = ev.n[H.pair][H.dir];
+    if (n_eval) atomicAdd(c, n_eval);
+    if (n_cost) atomicAdd(c + 1, n_cost);
+    if (n_glob) atomicAdd(c + 2, n_glob);
+}
+// every thread of the CTA, once all of its counts are in
+__device__ __forceinline__ void ev_flush(const EvCount& ev, const LvlBatch& B) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < B.n * 6; i += blockDim.x) {
+        const int pair = i / 6, dir = (i / 3) & 1, k = i % 3;
+        const unsigned v = ev.n[pair][dir][k];
+        if (v) atomicAdd(B.evals[pair] + (k == 2 ? 6 : 2 * k) + dir, (unsigned long long)v);
+    }
+}
+
 // Window slot of target centre (qx, qy): the word offset of its patch corner
 // from the window start in the low 16 bits, the index of its sum |b|^2 above;
 // -1 when the patch is not inside the staged window.
@@ -242,6 +279,10 @@ __device__ __forceinline__ int pr_slot(const RowGeom& G, const RowHdr& H, int P,
     }
 }
 
+// the gray int16 search reads its seeds as RowSeed, the others as RowRec
+template <int NCH, bool BITS> struct RecOf { typedef RowRec T; };
+template <> struct RecOf<2, false> { typedef RowSeed T; };
+
 // Producer warp p: stage the CTA's tiles n = p, p + PR_PROD, ... (launch tiles
 // blockIdx.x + n * gridDim.x) into buffer n mod nbuf.
 // NG = 0: one full and one empty mbarrier per buffer; every consumer warp
@@ -255,10 +296,11 @@ __device__ __forceinline__ int pr_slot(const RowGeom& G, const RowHdr& H, int P,
 template <int NCH, bool BITS, int NPROD, int NBUFMAX, int NG = 0>
 __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSched& S,
                            const RowMaps& TM, int buf_words, int nbuf, unsigned a_sm,
-                           RowRec (*rec)[PR_NACT], RowHdr* hdr, int* next, const RowGeom* geom,
-                           unsigned full0, unsigned empty0, volatile int* abort, long long limit,
-                           int pw, int lane) {
+                           typename RecOf<NCH, BITS>::T (*rec)[PR_NACT], RowHdr* hdr, int* next,
+                           const RowGeom* geom, unsigned full0, unsigned empty0, unsigned turn0,
+                           volatile int* abort, long long limit, int pw, int lane) {
     constexpr int PXW = px_words(NCH);
+    constexpr bool GRAY = NCH == 2 && !BITS;          // records as RowSeed
     int lastn[NBUFMAX];                      // the tile this warp last armed in each buffer
     int waits[NBUFMAX];                      // NG > 0: waits so far on this warp's empty barrier of b
 #pragma unroll
@@ -269,18 +311,6 @@ __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSch
         const int b = n % nbuf;
         const unsigned full = full0 + 8u * (NG > 0 ? (unsigned)(b * NG + n % NG) : (unsigned)b);
         const unsigned empty = empty0 + 8u * (NG > 0 ? (unsigned)(b * NPROD + pw) : (unsigned)b);
-        if (n >= nbuf) {            // the consumers released the buffer's last tile
-            const unsigned par = NG > 0 ? (unsigned)(waits[b]++) & 1u : (unsigned)((n / nbuf) - 1) & 1u;
-            const bool ok = __all_sync(FULL, mbar_wait(empty, par, limit, abort));
-            if (!ok) {
-                if (lane == 0 && !*abort) {
-                    for (int k = 0; k < B.n; ++k) atomicOr(B.err[k], (unsigned)PGM_ERR_TIMEOUT);
-                    *abort = 1;
-                }
-                break;
-            }
-        }
-        if (*abort) break;
         int lo = 0, hi = S.nk - 1;                   // slot holding tile t:
         while (lo < hi) {                            // the last k with cum[k] <= t
             const int mid = (lo + hi + 1) >> 1;
@@ -297,17 +327,6 @@ __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSch
         const int rbit = (rx0 + BORD) * NCH, rws = (rbit >> 5) & ~3;
         const int shr = BITS ? rbit - 32 * rws : PXW == 4 ? 0 : ((rx0 + BORD) & 3);
         const unsigned buf = a_sm + 4u * (unsigned)(b * buf_words);
-        fence_proxy_async();                         // the consumers' reads of this buffer come first
-        if (lane == 0) {                             // the reference region does not depend on the seeds
-            if constexpr (BITS) {                    // nonzero rows, then sign rows H + 2 BORD below
-                mbar_expect_tx(full, 8u * (unsigned)(G.bwr * G.ref_h));
-                tma2d(buf, &TM.m[k][0], rws, ry0 + BORD, full);
-                tma2d(buf + 4u * (unsigned)G.off_rs, &TM.m[k][0], rws, D.rh + 2 * BORD + ry0 + BORD, full);
-            } else {
-                mbar_expect_tx(full, 4u * (unsigned)(G.sp * G.ref_h));
-                tma2d(buf, &TM.m[k][0], PXW == 4 ? 2 * (rx0 + BORD) : rx0 + BORD - shr, ry0 + BORD, full);
-            }
-        }
         // the seed of this lane: active seed a = lane of the tile (Eq. 4 candidates, Eq. 5 draws)
         const int t4 = mc.t & 3;
         const int sx = (t4 == 0 || t4 == 3) ? 1 : -1, sy = (t4 == 0 || t4 == 2) ? 1 : -1;
@@ -407,38 +426,119 @@ __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSch
         R.w1 = R.nb1 != NO_CAND ? pr_slot<BITS>(G, H, P, R.px + lo16((uint32_t)R.nb1), R.py + hi16((uint32_t)R.nb1)) : -1;
         // the first two search candidates around the current match, the
         // centre of the search unless a propagated match wins
+        int nsearch = 0;
         if (R.s >= 0 && (R.f & F_VALID) && R.K > 0) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const uint32_t o = (uint32_t)(k ? R.r1 : R.r0);
                 const int qx = R.px + ux + lo16(o), qy = R.py + uy + hi16(o);
                 const bool ok = k < R.K && o != 0u && inside(D, qx, qy);
+                nsearch += ok;
                 const int w = ok ? pr_slot<BITS>(G, H, P, qx, qy) : -2;
                 if (k) R.wr1 = w; else R.wr0 = w;
             }
         }
-        rec[b][a] = R;
+        [[maybe_unused]] int at = 0, pend = 0;
+        if constexpr (GRAY) {
+            // the records lie in the order of their known candidates, most
+            // first: a consumer warp scores two neighbouring ones in step
+            pend = R.s < 0 ? 0
+                   : ((mc.refresh && (R.f & F_VALID)) ? 1 : 0) | (R.nb0 != NO_CAND ? 2 : 0) |
+                         (R.nb1 != NO_CAND ? 4 : 0) |
+                         (R.K <= 2 ? (R.wr0 != -2 ? 8 : 0) | (R.wr1 != -2 ? 16 : 0) : 0);
+            const int nc = __popc(pend & 7) + nsearch;
+            const unsigned below = (1u << lane) - 1u;
+            int more = 0;
+#pragma unroll
+            for (int v = 5; v >= 0; --v) {
+                const unsigned same = __ballot_sync(FULL, nc == v);
+                if (nc == v) at = more + __popc(same & below);
+                more += __popc(same);
+            }
+        }
+        // the buffer: only now is it waited for, so that it is held for the
+        // copies and the search, not for the reads of the seeds (a producer
+        // takes 4500 cycles for those; 9.43 -> 9.22 ms a colour step of 16
+        // pairs of 1024 x 436, 7.95 -> 7.54 ms a gray one).  With one
+        // empty barrier per buffer the tiles are staged in their order (the
+        // warp of tile n - 1 hands on the turn): a warp that looked at a
+        // buffer two tiles ahead would take the parity of the phase before
+        // for its own.
+        if (NG == 0 && n > 0) {
+            const unsigned par = (unsigned)(n / NPROD - (pw == 0)) & 1u;
+            if (!__all_sync(FULL, mbar_wait(turn0 + 8u * (unsigned)pw, par, limit, abort))) {
+                if (lane == 0 && !*abort) {
+                    for (int k = 0; k < B.n; ++k) atomicOr(B.err[k], (unsigned)PGM_ERR_TIMEOUT);
+                    *abort = 1;
+                }
+                break;
+            }
+        }
+        if (n >= nbuf) {            // the consumers released the buffer's last tile
+            const unsigned par = NG > 0 ? (unsigned)(waits[b]++) & 1u : (unsigned)((n / nbuf) - 1) & 1u;
+            const bool ok = __all_sync(FULL, mbar_wait(empty, par, limit, abort));
+            if (!ok) {
+                if (lane == 0 && !*abort) {
+                    for (int k = 0; k < B.n; ++k) atomicOr(B.err[k], (unsigned)PGM_ERR_TIMEOUT);
+                    *abort = 1;
+                }
+                break;
+            }
+        }
+        if (*abort) break;
+        fence_proxy_async();                         // the consumers' reads of this buffer come first
+        if (lane == 0) {
+            if constexpr (BITS) {                    // nonzero rows, then sign rows H + 2 BORD below
+                mbar_expect_tx(full, 8u * (unsigned)(G.bwr * G.ref_h));
+                tma2d(buf, &TM.m[k][0], rws, ry0 + BORD, full);
+                tma2d(buf + 4u * (unsigned)G.off_rs, &TM.m[k][0], rws, D.rh + 2 * BORD + ry0 + BORD, full);
+            } else {
+                mbar_expect_tx(full, 4u * (unsigned)(G.sp * G.ref_h));
+                tma2d(buf, &TM.m[k][0], PXW == 4 ? 2 * (rx0 + BORD) : rx0 + BORD - shr, ry0 + BORD, full);
+            }
+        }
+        if (lane == 0 && H.use_win) {
+            if constexpr (BITS) {
+                mbar_expect_tx(full, 8u * (unsigned)(G.bww * G.win_h));
+                tma2d(buf + 4u * (unsigned)G.off_win, &TM.m[k][1], wws, H.wy0 + BORD, full);
+                tma2d(buf + 4u * (unsigned)G.off_ws, &TM.m[k][1], wws,
+                      D.th + 2 * BORD + H.wy0 + BORD, full);
+            } else {
+                mbar_expect_tx(full, 4u * (unsigned)(G.sp * G.win_h) + 8u * (unsigned)(G.cwp * G.ch));
+                tma2d(buf + 4u * (unsigned)G.off_win, &TM.m[k][1],
+                      PXW == 4 ? 2 * (H.wx0 + BORD) : H.wx0 + BORD - H.shw, H.wy0 + BORD, full);
+                tma2d(buf + 4u * (unsigned)G.off_sb, &TM.m[k][2], H.wx0 + h - H.shs, H.wy0 + h, full);
+            }
+        }
+        if constexpr (!GRAY) {
+            rec[b][a] = R;
+        } else {
+            RowSeed Q;
+            Q.s = R.s;
+            Q.pxy = pack_u(R.px, R.py);
+            Q.roff = R.s < 0 ? 0 : (R.py - h - ry0) * G.sp + shr + (R.px - h - rx0) * PXW;
+            Q.fl = R.s < 0 ? 0 : R.f | (R.f0 << 8) | (pend << 16) | (R.K << 21);
+            Q.cost = R.cost;
+            Q.sa = R.sa;
+            Q.cand[0][0] = R.u;   Q.cand[0][1] = R.wu;
+            Q.cand[1][0] = R.nb0; Q.cand[1][1] = R.w0;
+            Q.cand[2][0] = R.nb1; Q.cand[2][1] = R.w1;
+            Q.cand[3][0] = pack_u(ux + lo16((uint32_t)R.r0), uy + hi16((uint32_t)R.r0));
+            Q.cand[3][1] = R.wr0;
+            Q.cand[4][0] = pack_u(ux + lo16((uint32_t)R.r1), uy + hi16((uint32_t)R.r1));
+            Q.cand[4][1] = R.wr1;
+            Q.r[0] = R.r0;
+            Q.r[1] = R.r1;
+            rec[b][at] = Q;
+        }
         if (lane == 0) {
             hdr[b] = H;
             next[b] = 0;
         }
         __syncwarp();
         if (lane == 0) {
-            if (H.use_win) {
-                if constexpr (BITS) {
-                    mbar_arrive_tx(full, 8u * (unsigned)(G.bww * G.win_h));
-                    tma2d(buf + 4u * (unsigned)G.off_win, &TM.m[k][1], wws, H.wy0 + BORD, full);
-                    tma2d(buf + 4u * (unsigned)G.off_ws, &TM.m[k][1], wws,
-                          D.th + 2 * BORD + H.wy0 + BORD, full);
-                } else {
-                    mbar_arrive_tx(full, 4u * (unsigned)(G.sp * G.win_h) + 8u * (unsigned)(G.cwp * G.ch));
-                    tma2d(buf + 4u * (unsigned)G.off_win, &TM.m[k][1],
-                          PXW == 4 ? 2 * (H.wx0 + BORD) : H.wx0 + BORD - H.shw, H.wy0 + BORD, full);
-                    tma2d(buf + 4u * (unsigned)G.off_sb, &TM.m[k][2], H.wx0 + h - H.shs, H.wy0 + h, full);
-                }
-            } else {
-                mbar_arrive(full);
-            }
+            mbar_arrive(full);
+            if (NG == 0) mbar_arrive(turn0 + 8u * (unsigned)((pw + 1) % NPROD));
         }
         lastn[b] = n;
     }
@@ -582,10 +682,10 @@ __device__ void pr_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
                            int buf_words, int nbuf, unsigned a_sm, const uint32_t* sm_gen,
                            RowRec (*rec)[PR_NACT], const RowHdr* hdr, int* next,
                            const RowGeom* geom, unsigned full0, unsigned empty0,
-                           volatile int* abort, long long limit, int lane) {
+                           volatile int* abort, long long limit, int lane, EvCount& ev) {
     constexpr int PXW = px_words(NCH), WPP = NCH / 2;
     constexpr int M = PC > 0 ? (PC * PC + 31) / 32 : (MAXP * MAXP) / 32;   // pixels per lane
-    static_assert(SP == 0 || (NCH == 6 && PC == 15), "fixed-pitch rows: six channels, P = 15");
+    static_assert(NCH == 6 && (SP == 0 || PC == 15), "six channels; fixed-pitch rows: P = 15");
     int cur_dir = -1, P = 0, h = 0;
     unsigned off[M];                 // byte offset of lane pixel m from a patch corner
     unsigned vmask = 0;              // bit m: lane pixel m lies in the patch
@@ -778,11 +878,7 @@ __device__ void pr_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
                 }
             }
         }
-        if (lane == 0) {
-            if (n_eval) atomicAdd(B.evals[H.pair] + H.dir, (unsigned long long)n_eval);
-            if (n_cost) atomicAdd(B.evals[H.pair] + 2 + H.dir, (unsigned long long)n_cost);
-            if (n_glob) atomicAdd(B.evals[H.pair] + 6 + H.dir, (unsigned long long)n_glob);
-        }
+        if (lane == 0) ev_add(ev, H, n_eval, n_cost, n_glob);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + 8u * b);         // this warp is done with the buffer
     }
@@ -799,14 +895,17 @@ k_pm_r(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     __shared__ RowRec s_rec[PR_NBUF][PR_NACT];
     __shared__ RowHdr s_hdr[PR_NBUF];
     __shared__ RowGeom s_geom[2];
-    __shared__ __align__(8) unsigned long long s_full[PR_NBUF], s_empty[PR_NBUF];
+    __shared__ __align__(8) unsigned long long s_full[PR_NBUF], s_empty[PR_NBUF], s_turn[PR_PROD];
     __shared__ int s_next[PR_NBUF];
     __shared__ int s_abort;
+    __shared__ EvCount s_ev;
     pdl_trigger();                  // the next phase may start its prologue
+    ev_clear(s_ev);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned a_sm = (unsigned)__cvta_generic_to_shared(sm);
     const unsigned full0 = (unsigned)__cvta_generic_to_shared(&s_full[0]);
     const unsigned empty0 = (unsigned)__cvta_generic_to_shared(&s_empty[0]);
+    const unsigned turn0 = (unsigned)__cvta_generic_to_shared(&s_turn[0]);
     if (threadIdx.x < 2)
         s_geom[threadIdx.x] = rg_geom(NCH, B.d[0][threadIdx.x].P, mc.sigma, mc.rs_W, mc.slack,
                                       mc.tile_w);
@@ -815,6 +914,7 @@ k_pm_r(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
             mbar_init(full0 + 8u * b, 1);
             mbar_init(empty0 + 8u * b, pr_cons(NCH, PC));
         }
+        for (int p = 0; p < PR_PROD; ++p) mbar_init(turn0 + 8u * p, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -823,10 +923,300 @@ k_pm_r(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     volatile int* abort = &s_abort;
     if (warp >= pr_cons(NCH, PC))
         pr_produce<NCH, false, PR_PROD, PR_NBUF>(B, mc, S, TM, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom, full0,
-                        empty0, abort, limit, warp - pr_cons(NCH, PC), lane);
+                        empty0, turn0, abort, limit, warp - pr_cons(NCH, PC), lane);
     else
         pr_consume<NCH, PC, SP>(B, mc, S, buf_words, nbuf, a_sm, sm, s_rec, s_hdr, s_next, s_geom,
-                            full0, empty0, abort, limit, lane);
+                            full0, empty0, abort, limit, lane, s_ev);
+    ev_flush(s_ev, B);
+}
+
+// ------------------------------------------------------------------
+// Gray search, two seeds per warp.  A gray patch is a fifth of the colour one's
+// loads and products, so with a warp per seed two thirds of the instructions
+// are the seed's and the candidate's bookkeeping; here each half-warp takes a
+// seed of its own and the two are scored in step (the producer sorts the
+// tile's seeds by their number of candidates, so the two have about as many:
+// 1.8 rounds a pair).  A tile's pairs go round the consumer warps in turn,
+// without a counter.  16 pairs of 1024 x 436: the two directions' search 8.1 ->
+// 7.0 ms, the step 8.05 -> 6.80 ms (level-0 phase 223 and 230 -> 185 and 165
+// us).  The same form for six channels (15 pixels and 45 reference words a
+// lane) was no faster than the warp per seed: 10.0 and 9.4 ms a step against
+// 9.2.
+//
+// Lane l of a half-warp holds the pixels l, l + 16, ... of the P x P patch in
+// raster order.
+template <int PC>
+struct GrayLane {
+    static constexpr int M = PC > 0 ? (PC * PC + 15) / 16 : (MAXP * MAXP) / 16;
+    unsigned off[M];                 // byte offsets from a patch corner
+    unsigned vmask;                  // bit m: lane pixel m lies in the patch
+    __device__ __forceinline__ void set(const RowGeom& G, int hl) {
+        const int P = PC > 0 ? PC : G.P;
+        int row = 0, col = hl;
+        while (col >= P) { col -= P; ++row; }
+        vmask = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const bool in = row < P;
+            off[m] = in ? 4u * (unsigned)(row * G.sp + col) : 0u;
+            vmask |= in ? 1u << m : 0u;
+            col += 16;
+            while (col >= P) { col -= P; ++row; }
+        }
+    }
+};
+
+// One staged tile, for one consumer warp: its share of the tile's pairs of
+// seeds (i0, i0 + NC, ...), a seed per half-warp.  Returns the warp's first
+// pair of the next tile.
+template <int PC, int NC>
+__device__ __forceinline__ int pg_tile(const LvlBatch& B, const MatchConst& mc, const RowGeom& G,
+                                       const RowHdr& H, const GrayLane<PC>& L, unsigned buf,
+                                       unsigned rec, int i0, int lane, EvCount& ev) {
+    constexpr int M = GrayLane<PC>::M;
+    const DirLvl& D = B.d[H.pair][H.dir];
+    const int P = PC > 0 ? PC : G.P, h = P / 2, hl = lane & 15, half = lane & 16;
+    const uint32_t* t32 = reinterpret_cast<const uint32_t*>(D.tgt);
+    const unsigned a_win = buf + 4u * (unsigned)G.off_win, a_sb = buf + 4u * (unsigned)G.off_sb;
+    const int sp = G.sp, cwp = G.cwp, tw = D.tw, th = D.th;
+    const int wx = H.wx0 + h, wy = H.wy0 + h, shw = H.shw, shs = H.shs;
+    const int limx = H.use_win ? G.win_w - P : -1, limy = G.win_h - P;
+    unsigned n_eval = 0, n_cost = 0, n_glob = 0;          // of this lane's seeds
+    int i = i0;
+    for (; i < PR_NACT / 2; i += NC) {
+        const unsigned a_rec = rec + (unsigned)sizeof(RowSeed) * (unsigned)(2 * i + (half >> 4));
+        const uint4 q0 = lds128(a_rec);
+        const int s = (int)q0.x, fl = (int)q0.w;
+        int pend = sd_pend(fl), K = sd_k(fl);
+        bool have = fl & F_VALID;
+        if (!have && pend == 0) K = 0;                    // nothing to score, no search
+        if (__any_sync(FULL, pend != 0 || K > 0)) {
+            const uint4 q1 = lds128(a_rec + 16u);
+            const int px = lo16(q0.y), py = (int)(q0.y >> 16);
+            const long long sa = (long long)((unsigned long long)q1.z | ((unsigned long long)q1.w << 32));
+            // candidates are compared by D - sum |a|^2 = sum |b|^2 - 2 <a, b>
+            long long bc = (long long)((unsigned long long)q1.x | ((unsigned long long)q1.y << 32)) - sa;
+            if (!have || mc.refresh) bc = LLONG_MAX;
+            // lane k < 5 holds candidate k: the current match (cost refresh),
+            // the two propagated ones (Eq. 4), the search around the match
+            const unsigned long long cd = lds64(a_rec + 32u + 8u * (unsigned)min(hl, 4));
+            int cu = (int)(uint32_t)cd, slot = (int)(uint32_t)(cd >> 32);
+            const int Ru = (int)lds32(a_rec + 32u);
+            int bu = Ru;
+            int ra[M];                       // reference words, zero for pixels past the patch
+            {
+                const bool rok = PGM_CHECK((int)q0.z >= 0 && (int)q0.z + (P - 1) * sp + P <= sp * G.ref_h,
+                                           B.err[H.pair]);
+                const unsigned base = buf + 4u * (rok ? q0.z : 0u);
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    // (pixel m of every lane lies in the patch for m < P^2 / 16)
+                    const int keep = (PC > 0 && m < (PC * PC) / 16) || ((L.vmask >> m) & 1u) ? -1 : 0;
+                    ra[m] = lds32(base + L.off[m]) & keep;
+                }
+            }
+            n_cost += pend & 1;
+            n_eval += __popc(pend & 6);               // the search's are counted once known
+            // the candidates in the paper's order, one per round
+            for (;;) {
+                const bool moved = K > 0 && (pend & 7) == 0 && (K > 2 || bu != Ru || !(fl & F_VALID));
+                if (__any_sync(FULL, moved)) {
+                    // a propagated match is the centre now (or the search has
+                    // more than two candidates):
+                    // the limited random search (Eq. 5) around the match held
+                    // after propagation: lane k holds candidate k < K
+                    bool ok = false;
+                    if (moved && have && hl < K) {
+                        int dx, dy;
+                        if (hl < 2) {
+                            const uint32_t o = (uint32_t)lds32(a_rec + 72u + 4u * (unsigned)hl);
+                            dx = lo16(o);
+                            dy = hi16(o);
+                        } else {
+                            const uint4 rq = philox(
+                                make_uint4((uint32_t)s,
+                                           ((uint32_t)B.visit << 16) | ((uint32_t)H.dir << 15) | (uint32_t)mc.t,
+                                           ((uint32_t)B.level << 16) | (uint32_t)(hl >> 1),
+                                           B.stream_id[H.pair]),
+                                mc.key0, mc.key1);
+                            dx = rs_off((hl & 1) ? rq.z : rq.x, hl, mc.rs_W, mc.rs_mode);
+                            dy = rs_off((hl & 1) ? rq.w : rq.y, hl, mc.rs_W, mc.rs_mode);
+                        }
+                        const int ux = lo16((uint32_t)bu) + dx, uy = hi16((uint32_t)bu) + dy;
+                        const int qx = px + ux, qy = py + uy;             // tested before packing
+                        ok = !(dx == 0 && dy == 0) && qx >= 0 && qy >= 0 && qx < tw && qy < th;
+                        cu = pack_u(ux, uy);
+                        const int x0 = qx - wx, y0 = qy - wy;
+                        slot = (unsigned)x0 <= (unsigned)limx && (unsigned)y0 <= (unsigned)limy && limx >= 0
+                                   ? (y0 * sp + shw + x0) | ((y0 * cwp + shs + x0) << 16) : -1;
+                    }
+                    const int found = (int)((__ballot_sync(FULL, ok) >> half) & 0xffffu);
+                    if (moved) pend = found;
+                }
+                if (K > 0 && (moved || (pend & 7) == 0)) {        // the search candidates are known
+                    K = 0;
+                    n_eval += __popc(pend);
+                }
+                if (!__any_sync(FULL, pend != 0)) break;
+                const bool ok = pend != 0;                // this seed has a candidate to score
+                const int c = half | ((__ffs(pend) - 1) & 15);
+                pend &= pend - 1;
+                const int xu = __shfl_sync(FULL, cu, c);
+                int xs = __shfl_sync(FULL, slot, c);
+                if (!ok) xs = 0;                          // (reads the window's corner)
+                int l[3] = {0, 0, 0}, hh[3] = {0, 0, 0};
+                long long sb = 0;
+                if (xs >= 0) {
+                    const bool in = PGM_CHECK(!ok || ((xs & 0xffff) + (P - 1) * sp + P <= sp * G.win_h &&
+                                                      (xs >> 16) < cwp * G.ch), B.err[H.pair]);
+                    if (!in) xs = 0;
+                    sb = (long long)lds64(a_sb + 8u * (unsigned)(xs >> 16));
+                    const unsigned base = a_win + 4u * (unsigned)(xs & 0xffff);
+#pragma unroll
+                    for (int m = 0; m < M; ++m) {
+                        const int v = lds32(base + L.off[m]);
+                        l[m % 3] = __dp2a_lo(v, ra[m], l[m % 3]);
+                        hh[m % 3] = __dp2a_hi(v, ra[m], hh[m % 3]);
+                    }
+                } else {
+                    // outside the window: from the padded image (pixels a lane
+                    // does not hold read the patch corner)
+                    const int qx = px + lo16((uint32_t)xu), qy = py + hi16((uint32_t)xu);
+                    if (PGM_CHECK(qx >= 0 && qy >= 0 && qx < tw && qy < th && h <= BORD,
+                                  B.err[H.pair])) {
+                        int row = 0, col = hl;
+                        while (col >= P) { col -= P; ++row; }
+#pragma unroll
+                        for (int m = 0; m < M; ++m) {
+                            const bool in = (L.vmask >> m) & 1u;
+                            const int v = (int)__ldg(t32 + (ptrdiff_t)(qy - h + (in ? row : 0)) * (D.tgt_pitch >> 1) +
+                                                     (qx - h + (in ? col : 0)));
+                            l[m % 3] = __dp2a_lo(v, ra[m], l[m % 3]);
+                            hh[m % 3] = __dp2a_hi(v, ra[m], hh[m % 3]);
+                            col += 16;
+                            while (col >= P) { col -= P; ++row; }
+                        }
+                        sb = (long long)D.sb2[(size_t)qy * D.sbp + qx];
+                    }
+                    ++n_glob;
+                }
+                __syncwarp();
+                const int tl = l[0] + l[1] + l[2], th_ = hh[0] + hh[1] + hh[2];
+                // sums over the half-warp: the low sums meet in lanes 0 .. 7, the
+                // high ones in lanes 8 .. 15
+                const bool up = hl & 8;
+                int v = (up ? th_ : tl) + __shfl_xor_sync(FULL, up ? tl : th_, 8);
+                v += __shfl_xor_sync(FULL, v, 4);
+                v += __shfl_xor_sync(FULL, v, 2);
+                v += __shfl_xor_sync(FULL, v, 1);
+                const int w = __shfl_xor_sync(FULL, v, 8);
+                const int sl = up ? w : v, sh = up ? v : w;
+                const long long cost = sb - 2ll * sl - 256ll * sh;
+                if (ok && cost < bc) {
+                    bc = cost;
+                    bu = xu;
+                    have = true;
+                }
+            }
+            if (hl == 0 && have && (mc.refresh || bu != Ru || !(fl & F_VALID))) {
+                D.u[s] = bu;
+                D.cost[s] = (unsigned long long)(bc + sa);
+                D.flags[s] = (uint8_t)((fl & 0xff) | F_VALID);
+            }
+        }
+        // the refresh dropped a match that found no successor
+        if (hl == 0 && !have && s >= 0 && (fl & 0xff) != ((fl >> 8) & 0xff)) D.flags[s] = (uint8_t)fl;
+    }
+    n_eval += __shfl_xor_sync(FULL, n_eval, 16);
+    n_cost += __shfl_xor_sync(FULL, n_cost, 16);
+    n_glob += __shfl_xor_sync(FULL, n_glob, 16);
+    if (lane == 0) ev_add(ev, H, n_eval, n_cost, n_glob);
+    return i - PR_NACT / 2;
+}
+
+// Consumer warps: every tile of the CTA in turn.  PF, PB > 0: the patch side
+// of the forward and the backward tiles (compile time), else at most MAXP
+// (run time).
+template <int PF, int PB>
+__device__ void pg_consume(const LvlBatch& B, const MatchConst& mc, const RowSched& S,
+                           int buf_words, int nbuf, unsigned a_sm, unsigned a_rec,
+                           const RowHdr* hdr, const RowGeom* geom, unsigned full0,
+                           unsigned empty0, volatile int* abort, long long limit, int warp,
+                           int lane, EvCount& ev) {
+    constexpr int NC = pr_cons(2, PF);
+    GrayLane<PF> lf;
+    GrayLane<PB> lb;
+    int cur_dir = -1, i0 = warp;
+    for (int n = 0;; ++n) {
+        const int t = blockIdx.x + n * gridDim.x;
+        if (t >= S.total) break;
+        const int b = n % nbuf;
+        if (!__all_sync(FULL, mbar_wait(full0 + 8u * b, (unsigned)(n / nbuf) & 1u, limit, abort))) {
+            if (lane == 0 && !*abort) {
+                for (int k = 0; k < B.n; ++k) atomicOr(B.err[k], (unsigned)PGM_ERR_TIMEOUT);
+                *abort = 1;
+            }
+            break;
+        }
+        const RowHdr H = hdr[b];
+        const unsigned buf = a_sm + 4u * (unsigned)(b * buf_words);
+        const unsigned rec = a_rec + (unsigned)(sizeof(RowSeed) * PR_NACT) * (unsigned)b;
+        if (PF == PB || H.dir == 0) {
+            if (PF != PB || PF == 0 ? H.dir != cur_dir : cur_dir < 0) lf.set(geom[H.dir], lane & 15);
+            i0 = pg_tile<PF, NC>(B, mc, geom[H.dir], H, lf, buf, rec, i0, lane, ev);
+        } else if constexpr (PF != PB) {
+            if (H.dir != cur_dir) lb.set(geom[H.dir], lane & 15);
+            i0 = pg_tile<PB, NC>(B, mc, geom[H.dir], H, lb, buf, rec, i0, lane, ev);
+        }
+        cur_dir = H.dir;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty0 + 8u * b);         // this warp is done with the buffer
+    }
+}
+
+template <int PF, int PB>
+__global__ void __launch_bounds__(32 * (PR_PROD + pr_cons(2, PF)), 1)
+k_pm_g(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_constant__ RowSched S,
+       const __grid_constant__ RowMaps TM, const int buf_words, const int nbuf,
+       const long long limit) {
+    extern __shared__ __align__(128) uint32_t sm[];
+    __shared__ RowSeed s_rec[PR_NBUF][PR_NACT];
+    __shared__ RowHdr s_hdr[PR_NBUF];
+    __shared__ RowGeom s_geom[2];
+    __shared__ __align__(8) unsigned long long s_full[PR_NBUF], s_empty[PR_NBUF], s_turn[PR_PROD];
+    __shared__ int s_next[PR_NBUF];
+    __shared__ int s_abort;
+    __shared__ EvCount s_ev;
+    pdl_trigger();                  // the next phase may start its prologue
+    ev_clear(s_ev);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned a_sm = (unsigned)__cvta_generic_to_shared(sm);
+    const unsigned full0 = (unsigned)__cvta_generic_to_shared(&s_full[0]);
+    const unsigned empty0 = (unsigned)__cvta_generic_to_shared(&s_empty[0]);
+    const unsigned turn0 = (unsigned)__cvta_generic_to_shared(&s_turn[0]);
+    if (threadIdx.x < 2)
+        s_geom[threadIdx.x] = rg_geom(2, B.d[0][threadIdx.x].P, mc.sigma, mc.rs_W, mc.slack,
+                                      mc.tile_w);
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < nbuf; ++b) {
+            mbar_init(full0 + 8u * b, 1);
+            mbar_init(empty0 + 8u * b, pr_cons(2, PF));
+        }
+        for (int p = 0; p < PR_PROD; ++p) mbar_init(turn0 + 8u * p, 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    pdl_wait();                     // the previous phase is complete and visible
+    volatile int* abort = &s_abort;
+    if (warp >= pr_cons(2, PF))
+        pr_produce<2, false, PR_PROD, PR_NBUF>(B, mc, S, TM, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom, full0,
+                        empty0, turn0, abort, limit, warp - pr_cons(2, PF), lane);
+    else
+        pg_consume<PF, PB>(B, mc, S, buf_words, nbuf, a_sm,
+                                (unsigned)__cvta_generic_to_shared(&s_rec[0][0]), s_hdr, s_geom,
+                                full0, empty0, abort, limit, warp, lane, s_ev);
+    ev_flush(s_ev, B);
 }
 
 // ------------------------------------------------------------------
@@ -844,7 +1234,7 @@ template <int NCH, int PC>
 __device__ void pr_consume_bits(const LvlBatch& B, const MatchConst& mc, const RowSched& S,
                                 int buf_words, int nbuf, unsigned a_sm, RowRec (*rec)[PR_NACT],
                                 const RowHdr* hdr, int* next, const RowGeom* geom, unsigned full0,
-                                unsigned empty0, volatile int* abort, long long limit, int lane) {
+                                unsigned empty0, volatile int* abort, long long limit, int lane, EvCount& ev) {
     constexpr int NR = NCH == 6 ? 3 : 1;          // aligned words per row and plane
     constexpr int NW = NR + 1;                    // staged words read per row and plane
     constexpr unsigned INF32 = 0xffffffffu;
@@ -1037,11 +1427,7 @@ __device__ void pr_consume_bits(const LvlBatch& B, const MatchConst& mc, const R
                 }
             }
         }
-        if (lane == 0) {
-            if (n_eval) atomicAdd(B.evals[H.pair] + H.dir, (unsigned long long)n_eval);
-            if (n_cost) atomicAdd(B.evals[H.pair] + 2 + H.dir, (unsigned long long)n_cost);
-            if (n_glob) atomicAdd(B.evals[H.pair] + 6 + H.dir, (unsigned long long)n_glob);
-        }
+        if (lane == 0) ev_add(ev, H, n_eval, n_cost, n_glob);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + 8u * b);
     }
@@ -1060,14 +1446,17 @@ k_pm_b(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     __shared__ RowRec s_rec[PB_NBUF][PR_NACT];
     __shared__ RowHdr s_hdr[PB_NBUF];
     __shared__ RowGeom s_geom[2];
-    __shared__ __align__(8) unsigned long long s_full[PB_NBUF], s_empty[PB_NBUF];
+    __shared__ __align__(8) unsigned long long s_full[PB_NBUF], s_empty[PB_NBUF], s_turn[PB_PROD];
     __shared__ int s_next[PB_NBUF];
     __shared__ int s_abort;
+    __shared__ EvCount s_ev;
     pdl_trigger();                  // the next phase may start its prologue
+    ev_clear(s_ev);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned a_sm = (unsigned)__cvta_generic_to_shared(sm);
     const unsigned full0 = (unsigned)__cvta_generic_to_shared(&s_full[0]);
     const unsigned empty0 = (unsigned)__cvta_generic_to_shared(&s_empty[0]);
+    const unsigned turn0 = (unsigned)__cvta_generic_to_shared(&s_turn[0]);
     if (threadIdx.x < 2)
         s_geom[threadIdx.x] = rg_geom_bits(NCH, B.d[0][threadIdx.x].P, mc.sigma, mc.rs_W, mc.slack,
                                            mc.tile_w);
@@ -1076,6 +1465,7 @@ k_pm_b(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
             mbar_init(full0 + 8u * b, 1);
             mbar_init(empty0 + 8u * b, PB_CONS);
         }
+        for (int p = 0; p < PB_PROD; ++p) mbar_init(turn0 + 8u * p, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -1084,11 +1474,12 @@ k_pm_b(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     volatile int* abort = &s_abort;
     if (warp >= PB_CONS)
         pr_produce<NCH, true, PB_PROD, PB_NBUF>(B, mc, S, TM, buf_words, nbuf, a_sm, s_rec, s_hdr,
-                                                s_next, s_geom, full0, empty0, abort, limit,
+                                                s_next, s_geom, full0, empty0, turn0, abort, limit,
                                                 warp - PB_CONS, lane);
     else
         pr_consume_bits<NCH, PC>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom,
-                                 full0, empty0, abort, limit, lane);
+                                 full0, empty0, abort, limit, lane, s_ev);
+    ev_flush(s_ev, B);
 }
 
 }  // namespace
@@ -1210,7 +1601,7 @@ template <int NCH, int PC>
 __device__ void ps_consume(const LvlBatch& B, const MatchConst& mc, const RowSched& S, int buf_words,
                            int nbuf, unsigned a_sm, RowRec (*rec)[PR_NACT], const RowHdr* hdr,
                            const RowGeom* geom, unsigned full0, unsigned empty0,
-                           volatile int* abort, long long limit, int cw, int lane) {
+                           volatile int* abort, long long limit, int cw, int lane, EvCount& ev) {
     constexpr unsigned INF32 = 0xffffffffu;
     const unsigned fac = mc.norm == PGM_L2SQ ? 2u : 1u;      // 4 = 1 << 2, 2 = 1 << 1
     int seen[PS_NBUF];                    // waits so far on this warp's full barrier of each buffer
@@ -1346,11 +1737,7 @@ __device__ void ps_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
         n_eval = __reduce_add_sync(FULL, n_eval);
         n_cost = __reduce_add_sync(FULL, n_cost);
         n_glob = __reduce_add_sync(FULL, n_glob);
-        if (lane == 0) {
-            if (n_eval) atomicAdd(B.evals[H.pair] + H.dir, (unsigned long long)n_eval);
-            if (n_cost) atomicAdd(B.evals[H.pair] + 2 + H.dir, (unsigned long long)n_cost);
-            if (n_glob) atomicAdd(B.evals[H.pair] + 6 + H.dir, (unsigned long long)n_glob);
-        }
+        if (lane == 0) ev_add(ev, H, n_eval, n_cost, n_glob);
         __syncwarp();
         if (lane == 0)                                         // the tile's buffer is free again
             mbar_arrive(empty0 + 8u * (unsigned)(b * PS_PROD + (n + nbuf) % PS_PROD));
@@ -1369,7 +1756,9 @@ k_pm_s(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     __shared__ __align__(8) unsigned long long s_full[PS_NBUF * PS_CONS], s_empty[PS_NBUF * PS_PROD];
     __shared__ int s_next[PS_NBUF];
     __shared__ int s_abort;
+    __shared__ EvCount s_ev;
     pdl_trigger();                  // the next phase may start its prologue
+    ev_clear(s_ev);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned a_sm = (unsigned)__cvta_generic_to_shared(sm);
     const unsigned full0 = (unsigned)__cvta_generic_to_shared(&s_full[0]);
@@ -1390,11 +1779,12 @@ k_pm_s(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     volatile int* abort = &s_abort;
     if (warp >= PS_CONS)
         pr_produce<NCH, true, PS_PROD, PS_NBUF, PS_CONS>(B, mc, S, TM, buf_words, nbuf, a_sm, s_rec, s_hdr,
-                                                s_next, s_geom, full0, empty0, abort, limit,
+                                                s_next, s_geom, full0, empty0, 0u, abort, limit,
                                                 warp - PS_CONS, lane);
     else
         ps_consume<NCH, PC>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_geom, full0, empty0,
-                            abort, limit, warp, lane);
+                            abort, limit, warp, lane, s_ev);
+    ev_flush(s_ev, B);
 }
 
 // Host side: launch configuration.  No device code below this line.
@@ -1577,7 +1967,9 @@ static RowMaps& pr_maps(const LvlBatch& B, int nch, bool bits, const RowSched& S
 // wait limit of the kernel's mbarrier waits (cycles); set by pgm_set_wait_limit
 long long wait_limit();
 
-template <int NCH, int PC, bool BITS = false, int SP = 0>
+// Colour (NCH = 6): one direction of patch side PF, staged row pitch PB (0: run
+// time); gray: patch sides of both directions; bit-planes: PF = PB = 0.
+template <int NCH, int PF, int PB, bool BITS = false>
 pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, const RowMaps& TM,
                     int buf_words, cudaStream_t st) {
     const int sms = device_sms();
@@ -1585,8 +1977,10 @@ pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, 
     // bit planes: one seed per lane once every consumer warp of a CTA has
     // tiles of its own, else the warp-per-seed form (coarse levels)
     const bool per_lane = BITS && S.total >= PS_CONS * sms;
-    auto kern = k_pm_r<NCH, PC, SP>;
-    if constexpr (BITS) kern = per_lane ? k_pm_s<NCH, PC> : k_pm_b<NCH, PC>;
+    void (*kern)(LvlBatch, MatchConst, RowSched, RowMaps, int, int, long long);
+    if constexpr (BITS) kern = per_lane ? k_pm_s<NCH, 0> : k_pm_b<NCH, 0>;
+    else if constexpr (NCH == 2) kern = k_pm_g<PF, PB>;
+    else kern = k_pm_r<NCH, PF, PB>;
     if (pgm_status r = smem_opt_in((const void*)kern); r != PGM_OK) return r;
     // the ring: as many buffers as fit beside the kernel's static shared
     // memory (the bit-plane kernel's tile records take about 33 KB)
@@ -1600,7 +1994,7 @@ pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, 
     while (nbuf < most && (nbuf + 1L) * buf_words * 4 <= cap) ++nbuf;
     const int smem = nbuf * buf_words * 4;
     const int grid = S.total < sms ? S.total : sms;       // one CTA per SM (shared memory)
-    const int threads = !BITS ? 32 * (PR_PROD + pr_cons(NCH, PC))
+    const int threads = !BITS ? 32 * (PR_PROD + pr_cons(NCH, PF))
                         : per_lane ? 32 * (PS_PROD + PS_CONS) : 32 * (PB_PROD + PB_CONS);
     PGM_TRY(launch_pdl(kern, dim3(grid), dim3(threads), smem, st, B, mc, S, TM, buf_words, nbuf,
                        wait_limit()),
@@ -1609,22 +2003,36 @@ pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, 
 }
 
 // The consumer specialisation of a direction's patch side: compile-time sides
-// for the common 6-channel patches (15, 11) and 2-channel ones (15, 11, 8),
-// else the run-time form.
+// for the common patches (15, 11; gray also 8), else the run-time form.
 template <int NCH>
 pgm_status launch_dir(const LvlBatch& B, const MatchConst& mc, const RowSched& S, const RowGeom& G,
                       const RowMaps& TM, int buf_words, cudaStream_t st) {
     const int P = G.P;
-    // fixed-pitch rows: their one-past reads must land in the next region
-    if constexpr (NCH == 6)
+    if constexpr (NCH == 6) {
+        // fixed-pitch rows: their one-past reads must land in the next region
         if (P == 15 && G.sp == PR_ROWS_SP && G.pxw == 4 && G.off_win >= G.sp * G.ref_h &&
             G.off_sb - G.off_win >= G.sp * G.win_h && G.words - G.off_sb >= G.sp + 4 * (P + 2) &&
             G.sp / 4 >= G.win_w + 2)
-            return launch_r<NCH, 15, false, PR_ROWS_SP>(B, mc, S, TM, buf_words, st);
-    if (P == 15) return launch_r<NCH, 15>(B, mc, S, TM, buf_words, st);
-    if (P == 11) return launch_r<NCH, 11>(B, mc, S, TM, buf_words, st);
-    if (NCH == 2 && P == 8) return launch_r<NCH, 8>(B, mc, S, TM, buf_words, st);
-    return launch_r<NCH, 0>(B, mc, S, TM, buf_words, st);
+            return launch_r<6, 15, PR_ROWS_SP>(B, mc, S, TM, buf_words, st);
+        if (P == 15) return launch_r<6, 15, 0>(B, mc, S, TM, buf_words, st);
+        if (P == 11) return launch_r<6, 11, 0>(B, mc, S, TM, buf_words, st);
+        return launch_r<6, 0, 0>(B, mc, S, TM, buf_words, st);
+    } else {
+        if (P == 15) return launch_r<2, 15, 15>(B, mc, S, TM, buf_words, st);
+        if (P == 11) return launch_r<2, 11, 11>(B, mc, S, TM, buf_words, st);
+        if (P == 8) return launch_r<2, 8, 8>(B, mc, S, TM, buf_words, st);
+        return launch_r<2, 0, 0>(B, mc, S, TM, buf_words, st);
+    }
+}
+
+// Both directions in one launch.
+template <int NCH>
+pgm_status launch_both(const LvlBatch& B, const MatchConst& mc, const RowSched& S, const RowGeom* G,
+                       const RowMaps& TM, int buf_words, cudaStream_t st) {
+    if constexpr (NCH == 2) {
+        if (G[0].P == G[1].P) return launch_dir<2>(B, mc, S, G[0], TM, buf_words, st);
+    }
+    return launch_r<NCH, 0, 0>(B, mc, S, TM, buf_words, st);
 }
 
 bool pm_tile_fits(const LvlBatch& B, const MatchConst& mc, int nch) {
@@ -1662,10 +2070,10 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
         *nlaunch = 1;
         RowMaps& TM = pr_maps(B, nch, bits, S[2], G);
         if (bits)
-            return nch == 2 ? launch_r<2, 0, true>(B, mc, S[2], TM, words, st)
-                            : launch_r<6, 0, true>(B, mc, S[2], TM, words, st);
-        return nch == 2 ? launch_r<2, 0>(B, mc, S[2], TM, words, st)
-                        : launch_r<6, 0>(B, mc, S[2], TM, words, st);
+            return nch == 2 ? launch_r<2, 0, 0, true>(B, mc, S[2], TM, words, st)
+                            : launch_r<6, 0, 0, true>(B, mc, S[2], TM, words, st);
+        return nch == 2 ? launch_both<2>(B, mc, S[2], G, TM, words, st)
+                        : launch_both<6>(B, mc, S[2], G, TM, words, st);
     }
     for (int d = 0; d < 2; ++d) {
         if (S[d].total == 0) continue;
@@ -1673,8 +2081,8 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
         const cudaStream_t sd = d == 1 && st2 ? st2 : st;
         pgm_status r;
         if (bits)          // the bit-plane consumer's inner loops do not depend on P
-            r = nch == 2 ? launch_r<2, 0, true>(B, mc, S[d], TM, G[d].words, sd)
-                         : launch_r<6, 0, true>(B, mc, S[d], TM, G[d].words, sd);
+            r = nch == 2 ? launch_r<2, 0, 0, true>(B, mc, S[d], TM, G[d].words, sd)
+                         : launch_r<6, 0, 0, true>(B, mc, S[d], TM, G[d].words, sd);
         else
             r = nch == 2 ? launch_dir<2>(B, mc, S[d], G[d], TM, G[d].words, sd)
                          : launch_dir<6>(B, mc, S[d], G[d], TM, G[d].words, sd);
