@@ -721,12 +721,13 @@ pgm_status launch_cost_fill(const LvlBatch& B, const MatchConst& mc, int nch, in
     if (max_seeds <= 0) return PGM_OK;
     KScope ks(PGM_K_COST, st);
     dim3 g((max_seeds + 7) / 8, 2, B.n);
-    if (mc.norm == PGM_L2SQ) {
+    // the staged kernels take the bit-planes under either cost
+    if (mc.norm == PGM_L2SQ || mc.descriptor == PGM_DIR) {
         bool handled = false;
         pgm_status r = launch_cost_tile(B, mc, nch, &handled, st);
         if (r != PGM_OK || handled) return r;
-        PGM_DISPATCH_X(k_cost_x, g, B, mc);
     }
+    if (mc.norm == PGM_L2SQ) PGM_DISPATCH_X(k_cost_x, g, B, mc);
     else PGM_DISPATCH_NCH_PPL_NORM(k_cost, g, B, mc);
     return last_status();
 }
@@ -736,15 +737,15 @@ pgm_status launch_pm_phase(const LvlBatch& B, const MatchConst& mc, int nch, int
     if (max_seeds <= 0) return PGM_OK;
     KScope ks(PGM_K_PM, st);
     dim3 g((max_seeds + 7) / 8, 2, B.n);   // max_seeds: half-row width x rows
-    if (mc.norm == PGM_L2SQ) {
+    if (mc.norm == PGM_L2SQ || mc.descriptor == PGM_DIR) {
         bool handled = false;
         int nl = 0;
         pgm_status r = launch_pm_tile(B, mc, nch, maxP, &nl, &handled, st, st2);
         if (handled) ks.n = nl;
         if (r != PGM_OK || handled) return r;
         if (mc.refresh) return PGM_ERR_UNSUPPORTED;     // the per-seed kernel does no refresh
-        PGM_DISPATCH_X(k_pm_x, g, B, mc);
     }
+    if (mc.norm == PGM_L2SQ) PGM_DISPATCH_X(k_pm_x, g, B, mc);
     else PGM_DISPATCH_NCH_PPL_NORM(k_pm, g, B, mc);
     return last_status();
 }
