@@ -288,6 +288,9 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
                           bool* handled, cudaStream_t st, cudaStream_t st2);
 pgm_status launch_cost_tile(const LvlBatch& B, const MatchConst& mc, int nch, bool* handled,
                             cudaStream_t st);
+// pm_direct.cu: the search phases of few seeds, a warp per seed and no staging
+bool pm_direct_fits(const LvlBatch& B, const MatchConst& mc, int nch, int sms);
+pgm_status launch_pm_direct(const LvlBatch& B, const MatchConst& mc, int nch, cudaStream_t st);
 // filter.cu
 struct FiltItem {                 // the level-0 forward field of one pair
     const uint8_t* flags;

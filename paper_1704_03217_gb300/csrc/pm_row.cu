@@ -2045,7 +2045,8 @@ bool pm_tile_fits(const LvlBatch& B, const MatchConst& mc, int nch) {
 bool pm_tile_split(const LvlBatch& B, const MatchConst& mc, int nch) {
     RowSched S[3];
     RowGeom G[2];
-    return pr_plan(B, mc, nch, S, G) && (S[2].total > device_sms() || 2 * B.n > PR_MAPS);
+    return pr_plan(B, mc, nch, S, G) && !pm_direct_fits(B, mc, nch, device_sms()) &&
+           (S[2].total > device_sms() || 2 * B.n > PR_MAPS);
 }
 
 // *handled = false when pr_plan refuses the batch; the caller then uses the
@@ -2064,6 +2065,10 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
     if (!pr_plan(B, mc, nch, S, G)) return PGM_OK;
     *handled = true;
     if (S[2].total == 0) return PGM_OK;
+    if (pm_direct_fits(B, mc, nch, device_sms())) {
+        *nlaunch = 1;
+        return launch_pm_direct(B, mc, nch, st);
+    }
     const bool bits = use_bits(mc);
     if (S[2].total <= device_sms() && 2 * B.n <= PR_MAPS) {
         const int words = G[0].words > G[1].words ? G[0].words : G[1].words;
