@@ -248,7 +248,11 @@ struct PyrItem {                  // one image in one pyramid launch
     int brow;                     // words per bit-plane row
     int pad2;
 };
-struct PyrBatch { int n; int pad; PyrItem it[PYR_MAXB]; };
+struct PyrBatch {
+    int n; int pad;
+    PyrItem it[PYR_MAXB];
+    int cum[PYR_MAXB + 1];        // launches over all levels: the items' first blocks
+};
 pgm_status launch_pyramid_batch(const pgm_params* p, int n, const PyrPlan* plans,
                                 const uint8_t* const* imgs, const int* cs, const size_t* pitches,
                                 uint8_t* const* pyrs, cudaStream_t st);

@@ -21,8 +21,21 @@ __device__ __forceinline__ int gray_q14(int r, int g, int b) {
     return (4899 * r + 9617 * g + 1868 * b + 8192) >> 14;
 }
 
-// Every kernel takes a batch of images (blockIdx.z); the grid covers the
-// largest image and blocks outside an image's extent return.
+// Level 0 and the downsampling take a batch of images (blockIdx.z); the grid
+// covers the largest image and blocks outside an image's extent return.  The
+// colour conversion, the gradients and the bit-planes depend only on the
+// level images: one launch takes every level and direction of every image,
+// its blocks numbered through (PyrBatch::cum), where a launch per level and
+// direction left the chip to a few small blocks at a time (two frames of 1920 x
+// 1080: 22 -> 7 launches).
+__device__ __forceinline__ int pyr_item(const PyrBatch& B, int block) {
+    int lo = 0, hi = B.n - 1;                 // the last item with cum <= block
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (B.cum[mid] <= block) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
 
 // ---------------------------------------------------------------- level 0
 // mode 0: gray input copied; mode 1: RGB -> gray; mode 2: RGB -> 3 planes.
@@ -113,34 +126,27 @@ __device__ __forceinline__ uint32_t icbrt48(unsigned long long v) {
 }
 
 // CIELab companding function of t = T / (255 * 2^16), result scaled by 2^16.
-__device__ __forceinline__ long long lab_f(long long T) {
-    if (T * 24389 > 216LL * 255 * 65536) {               // t > (6/29)^3
-        // t * 2^48 = floor(T 2^32 / 255) = T (2^32 - 1) / 255 + floor(T / 255)
-        const uint32_t t32 = (uint32_t)T;                 // T < 2^24
-        const unsigned long long V = (unsigned long long)t32 * 16843009ull + t32 / 255u;
-        return (long long)icbrt48(V);
+__device__ __forceinline__ int lab_f(uint32_t T) {
+    if (T > 148006u) {                                    // t > (6/29)^3: T 24389 > 216 255 2^16
+        // t * 2^48 = floor(T 2^32 / 255) = T (2^32 - 1) / 255 + floor(T / 255); T < 2^24
+        return (int)icbrt48((unsigned long long)T * 16843009ull + T / 255u);
     }
-    long long num = T * (841 * 29) + 4LL * 65536 * 108 * 255;          // t * 841/108 + 4/29
-    return num / (108LL * 255 * 29);                                    // num > 0
-}
-
-__device__ __forceinline__ long long fdiv(long long a, long long b) {  // floor, b > 0
-    long long q = a / b;
-    return (a % b != 0 && a < 0) ? q - 1 : q;
+    // t * 841/108 + 4/29
+    return (int)(((unsigned long long)T * (841 * 29) + 4ull * 65536 * 108 * 255) / (108u * 255 * 29));
 }
 
 __device__ __forceinline__ void to_lab(int r, int g, int b, int* o) {
     // D65 RGB -> XYZ / white, Q16 rows summing to 65536, linear RGB
-    long long X = 28439LL * r + 24656LL * g + 12441LL * b;
-    long long Y = 13937LL * r + 46869LL * g + 4730LL * b;
-    long long Z = 1164LL * r + 7175LL * g + 57197LL * b;
-    long long fx = lab_f(X), fy = lab_f(Y), fz = lab_f(Z);
-    long long Ls = fdiv((116 * fy - 16 * 65536) * 255 + 3276800, 6553600);
-    long long As = (500 * (fx - fy) + 128 * 65536 + 32768) >> 16;      // floor division
-    long long Bs = (200 * (fy - fz) + 128 * 65536 + 32768) >> 16;
-    o[0] = clampi((int)Ls, 0, 255);
-    o[1] = clampi((int)As, 0, 255);
-    o[2] = clampi((int)Bs, 0, 255);
+    const int fx = lab_f(28439u * r + 24656u * g + 12441u * b);
+    const int fy = lab_f(13937u * r + 46869u * g + 4730u * b);
+    const int fz = lab_f(1164u * r + 7175u * g + 57197u * b);
+    // 9039 <= f <= 65536: the numerator lies in [3263540, 1674444800]
+    const int Ls = (int)((uint32_t)((116 * fy - 16 * 65536) * 255 + 3276800) / 6553600u);
+    const int As = (500 * (fx - fy) + 128 * 65536 + 32768) >> 16;      // floor division
+    const int Bs = (200 * (fy - fz) + 128 * 65536 + 32768) >> 16;
+    o[0] = clampi(Ls, 0, 255);
+    o[1] = clampi(As, 0, 255);
+    o[2] = clampi(Bs, 0, 255);
 }
 
 __device__ __forceinline__ void to_ycrcb(int r, int g, int b, int* o) {
@@ -150,18 +156,30 @@ __device__ __forceinline__ void to_ycrcb(int r, int g, int b, int* o) {
     o[2] = clampi(((b - y) * 9241 + (128 << 14) + 8192) >> 14, 0, 255);
 }
 
-__global__ void k_convert(const __grid_constant__ PyrBatch B) {
-    const PyrItem& it = B.it[blockIdx.z];
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
+// Four consecutive pixels per thread, one 32-bit access per plane (level rows
+// are padded to 16 bytes; the pad is converted too and never read).
+constexpr int CV_W = 128, CV_H = 8;           // pixels of a block
+__global__ void __launch_bounds__(256) k_convert(const __grid_constant__ PyrBatch B) {
+    const int k = pyr_item(B, blockIdx.x);
+    const PyrItem& it = B.it[k];
+    const int nbx = (it.sw + CV_W - 1) / CV_W, at = (int)blockIdx.x - B.cum[k];
+    const int x = (at % nbx) * CV_W + 4 * (int)(threadIdx.x & 31), y = (at / nbx) * CV_H + (int)(threadIdx.x >> 5);
     if (x >= it.sw || y >= it.sh) return;
     const size_t o = (size_t)y * it.srow + x, plane = it.splane;
-    int r = it.src[o], g = it.src[plane + o], b = it.src[2 * plane + o];
-    int v[3];
-    if (it.mode == SP_LAB) to_lab(r, g, b, v); else to_ycrcb(r, g, b, v);
-    it.dst[o] = (uint8_t)v[0];
-    it.dst[plane + o] = (uint8_t)v[1];
-    it.dst[2 * plane + o] = (uint8_t)v[2];
+    const uint32_t r = *reinterpret_cast<const uint32_t*>(it.src + o);
+    const uint32_t g = *reinterpret_cast<const uint32_t*>(it.src + plane + o);
+    const uint32_t b = *reinterpret_cast<const uint32_t*>(it.src + 2 * plane + o);
+    uint32_t c[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int R = (r >> (8 * i)) & 255, G = (g >> (8 * i)) & 255, Bl = (b >> (8 * i)) & 255;
+        int v[3];
+        if (it.mode == SP_LAB) to_lab(R, G, Bl, v); else to_ycrcb(R, G, Bl, v);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) c[q] |= (uint32_t)v[q] << (8 * i);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint32_t*>(it.dst + q * plane + o) = c[q];
 }
 
 // ----------------------------------------------------------------- Sobel
@@ -173,9 +191,8 @@ __global__ void k_convert(const __grid_constant__ PyrBatch B) {
 // x, both within int16) are kept per input row as one packed word, and the
 // vertical passes finish Gx and Gy (separable and exact in integers).  The
 // output words (px_words per pixel: 3 data words and a zero word for colour,
-// one word for gray) are staged in shared memory and leave as contiguous
-// 16-byte stores, one tile row of each output array at a time.  A block at an
-// image edge also writes the replicated border of BORD pixels next to it (a
+// one word for gray) leave as one 16-byte store per colour pixel.  A block at an
+// image edge stages them in shared memory and also writes the replicated border of BORD pixels next to it (a
 // border pixel repeats the descriptor of the nearest image pixel, which the
 // block holds), so every patch with its centre in the image can be read
 // without clamping.
@@ -186,6 +203,14 @@ __device__ __forceinline__ int sb_d(int S, int i) {
 __device__ __forceinline__ int sb_s(int S, int i) {
     return S == 5 ? (i == 0 ? 1 : i == 1 ? 4 : i == 2 ? 6 : i == 3 ? 4 : 1) : (i == 1 ? 2 : 1);
 }
+// two values split into signed bytes (match_common.cuh, split_bytes) on packed
+// halves: t = a + 64 + 2^14 >= 0 per half holds a_l + 64 in its low 7 bits and
+// a_h + 128 above
+__device__ __forceinline__ uint32_t sb_split(int a0, int a1) {
+    const uint32_t t = (uint32_t)(a0 + 16448) + ((uint32_t)(a1 + 16448) << 16);
+    const uint32_t l = (t & 0x007f007fu) + 0x00c000c0u, h = (t >> 7) & 0x01ff01ffu;   // + 256, + 128
+    return __byte_perm(l, h, 0x6420) ^ 0x80800000u;
+}
 template <int S, int C>
 __global__ void __launch_bounds__(SB_TW * SB_TY) k_sobel(const __grid_constant__ PyrBatch B,
                                                          int dir_only) {
@@ -195,12 +220,13 @@ __global__ void __launch_bounds__(SB_TW * SB_TY) k_sobel(const __grid_constant__
     constexpr int PXW = px_words(2 * C);                 // words per pixel in the output arrays
     constexpr int OW = SB_TW * PXW;                      // output words per tile row and array
     __shared__ __align__(16) uint8_t sI[C][IH][IW];      // column c holds x = x0 - SB_XO + c
-    __shared__ uint32_t sH[C][IH][SB_TW];                // (sum d v) low 16, (sum s v) high 16
+    __shared__ __align__(16) uint32_t sH[C][IH][SB_TW];  // (sum d v) low 16, (sum s v) high 16
     __shared__ __align__(16) uint32_t sO[2][SB_TH][OW];  // descriptor words, split words
-    const PyrItem& it = B.it[blockIdx.z];
+    const int item = pyr_item(B, blockIdx.x);
+    const PyrItem& it = B.it[item];
     const int w = it.sw, h = it.sh, row = it.srow;
-    const int x0 = blockIdx.x * SB_TW, y0 = blockIdx.y * SB_TH;
-    if (x0 >= w || y0 >= h) return;                     // the whole block (uniform)
+    const int nbx = (w + SB_TW - 1) / SB_TW, at = (int)blockIdx.x - B.cum[item];
+    const int x0 = (at % nbx) * SB_TW, y0 = (at / nbx) * SB_TH;
     const size_t plane = it.splane;
     const uint8_t* in = it.src;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * SB_TW + tx;
@@ -222,18 +248,32 @@ __global__ void __launch_bounds__(SB_TW * SB_TY) k_sobel(const __grid_constant__
         }
     }
     __syncthreads();
-    for (int r = ty; r < IH; r += SB_TY)
+    // four neighbouring outputs from three words
+    for (int e = tid; e < C * IH * (SB_TW / 4); e += NT) {
+        const int ch = e / (IH * (SB_TW / 4)), rem = e - ch * (IH * (SB_TW / 4));
+        const int r = rem / (SB_TW / 4), q = rem - r * (SB_TW / 4);
+        const uint32_t* wd = reinterpret_cast<const uint32_t*>(&sI[ch][r][4 * q]);   // x0 + 4 q - 4 ..
+        int v[12];
 #pragma unroll
-        for (int ch = 0; ch < C; ++ch) {
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t u = wd[k];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[4 * k + i] = (int)((u >> (8 * i)) & 255u);
+        }
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
             int sd = 0, ss = 0;
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                const int v = sI[ch][r][SB_XO - R + tx + i];
-                sd += sb_d(S, i) * v;
-                ss += sb_s(S, i) * v;
+            for (int t = 0; t < S; ++t) {
+                const int z = v[SB_XO - R + i + t];
+                sd += sb_d(S, t) * z;
+                ss += sb_s(S, t) * z;
             }
-            sH[ch][r][tx] = (uint32_t)(uint16_t)sd | ((uint32_t)ss << 16);
+            o[i] = (uint32_t)(uint16_t)sd | ((uint32_t)ss << 16);
         }
+        *reinterpret_cast<uint4*>(&sH[ch][r][4 * q]) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
     __syncthreads();
     int g[2][2 * C];
 #pragma unroll
@@ -266,39 +306,50 @@ __global__ void __launch_bounds__(SB_TW * SB_TY) k_sobel(const __grid_constant__
             g[k][C + ch] = b2;
         }
     }
-    // pixel-interleaved int16 as 32-bit words (2C is even), and the same
-    // words with every value a split into signed bytes a = 128 a_h + a_l
-    // (a_l in [-64, 63]) for the dp2a cross products
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-#pragma unroll
-        for (int q = 0; q < PXW; ++q) {
-            const bool dw = q < C;
-            sO[0][2 * ty + k][tx * PXW + q] =
-                dw ? (uint32_t)(uint16_t)g[k][2 * q] | ((uint32_t)(uint16_t)g[k][2 * q + 1] << 16) : 0u;
-            sO[1][2 * ty + k][tx * PXW + q] = dw ? (uint32_t)split_bytes(g[k][2 * q], g[k][2 * q + 1]) : 0u;
-        }
-    __syncthreads();
     // dst and split point at pixel (0, 0) of padded arrays with rows of rw
-    // words (a multiple of 4); pixel (x, y) starts at word y rw + x PXW, and
-    // x0 PXW is a multiple of 32 words, so tile rows are 16-byte aligned
+    // words (a multiple of 4); pixel (x, y) starts at word y rw + x PXW
     const ptrdiff_t rw = (ptrdiff_t)(it.drow >> 1);
     uint32_t* const dst0 = reinterpret_cast<uint32_t*>(it.dst);
     uint32_t* const dst1 = it.split;
     // this block's output: its tile, widened by the border where it touches
     // an image edge
     const bool left = x0 == 0, right = x0 + SB_TW >= w, top = y0 == 0, bottom = y0 + SB_TH >= h;
+    const bool edge = left || right || top || bottom;
     const int xa = left ? -BORD : x0, xb = right ? w + BORD : x0 + SB_TW;
     const int ya = top ? -BORD : y0, yb = bottom ? h + BORD : y0 + SB_TH;
-    if (!(left || right || top || bottom)) {
-        constexpr int NQ = OW / 4;
-        for (int e = tid; e < 2 * SB_TH * NQ; e += NT) {
-            const int a = e / (SB_TH * NQ), rem = e - a * (SB_TH * NQ), r = rem / NQ, q = rem - r * NQ;
-            const uint4 v = *reinterpret_cast<const uint4*>(&sO[a][r][4 * q]);
-            *reinterpret_cast<uint4*>((a ? dst1 : dst0) + (ptrdiff_t)(y0 + r) * rw +
-                                      (ptrdiff_t)x0 * PXW + 4 * q) = v;
+    // pixel-interleaved int16 as 32-bit words (2C is even), and the same
+    // words with every value a split into signed bytes a = 128 a_h + a_l
+    // (a_l in [-64, 63]) for the dp2a cross products.  A block inside the image
+    // stores its pixels at once (a warp's row is contiguous); one at an edge
+    // stages them for the border.
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        uint32_t wv[PXW], sv[PXW];
+#pragma unroll
+        for (int q = 0; q < PXW; ++q) {
+            const bool dw = q < C;
+            wv[q] = dw ? (uint32_t)(uint16_t)g[k][2 * q] | ((uint32_t)(uint16_t)g[k][2 * q + 1] << 16) : 0u;
+            sv[q] = dw ? sb_split(g[k][2 * q], g[k][2 * q + 1]) : 0u;
         }
-    } else {
+        if (!edge) {
+            const ptrdiff_t o = (ptrdiff_t)(y0 + 2 * ty + k) * rw + (ptrdiff_t)(x0 + tx) * PXW;
+            if constexpr (PXW == 4) {
+                *reinterpret_cast<uint4*>(dst0 + o) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+                *reinterpret_cast<uint4*>(dst1 + o) = make_uint4(sv[0], sv[1], sv[2], sv[3]);
+            } else {
+                dst0[o] = wv[0];
+                dst1[o] = sv[0];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < PXW; ++q) {
+                sO[0][2 * ty + k][tx * PXW + q] = wv[q];
+                sO[1][2 * ty + k][tx * PXW + q] = sv[q];
+            }
+        }
+    }
+    if (edge) {
+        __syncthreads();
         // a border pixel takes the words of the nearest image pixel, which
         // lies in this tile; a warp walks one output row, a pixel per lane
         // (colour pixels as one 16-byte store)
@@ -325,12 +376,14 @@ __global__ void __launch_bounds__(SB_TW * SB_TY) k_sobel(const __grid_constant__
 // For the direction descriptor: word w of padded row yy of the nonzero and
 // the sign bit-plane from the padded descriptor (bit b = x nch + c holds
 // value c of padded pixel x; words past the row are zero).  One thread per
-// word of one image (blockIdx.z).
+// word.
 template <int NCH>
 __global__ void k_bits(const __grid_constant__ PyrBatch B) {
     constexpr int PXE = 2 * px_words(NCH);       // int16 elements per padded pixel
-    const PyrItem& it = B.it[blockIdx.z];
-    const int w = blockIdx.x * blockDim.x + threadIdx.x, yy = blockIdx.y * blockDim.y + threadIdx.y;
+    const int item = pyr_item(B, blockIdx.x);
+    const PyrItem& it = B.it[item];
+    const int nbx = (it.brow + 31) / 32, at = (int)blockIdx.x - B.cum[item];
+    const int w = (at % nbx) * 32 + threadIdx.x, yy = (at / nbx) * 8 + threadIdx.y;
     const int pw = it.sw + 2 * BORD, ph = it.sh + 2 * BORD;
     if (w >= it.brow || yy >= ph) return;
     // padded pixel x of row yy: it.dst points at pixel (0, 0), rows drow int16
@@ -376,11 +429,7 @@ pgm_status launch_pyramid_batch(const pgm_params* p, int n, const PyrPlan* plans
     const int dir_only = p->descriptor;      // 0 full, 1 signs, 2 sectors
     for (int base = 0; base < n; base += PYR_MAXB) {
         const int m = n - base < PYR_MAXB ? n - base : PYR_MAXB;
-        int nlaunch = L + nsch * L * (dir_only == 1 ? 2 : 1);
-        for (int s = 0; s < nsch; ++s)
-            for (int l = 0; l < L; ++l)
-                nlaunch += p0.space[s][l] == SP_LAB || p0.space[s][l] == SP_YCRCB;
-        KScope ks(PGM_K_PYRAMID, st, nlaunch);
+        KScope ks(PGM_K_PYRAMID, st, L);
         // level 0
         int mw = 0, mh = 0;
         memset(&B, 0, sizeof(B));
@@ -410,56 +459,67 @@ pgm_status launch_pyramid_batch(const pgm_params* p, int n, const PyrPlan* plans
             }
             k_down<<<grid(mw, mh, m * C), blk, 0, st>>>(B, C);
         }
-        for (int s = 0; s < nsch; ++s)
-            for (int l = 0; l < L; ++l) {
-                const int sp = p0.space[s][l];
-                mw = mh = 0;
-                for (int k = 0; k < m; ++k) {
-                    const PyrPlan& pp = plans[base + k];
-                    mw = pp.W[l] > mw ? pp.W[l] : mw; mh = pp.H[l] > mh ? pp.H[l] : mh;
-                }
-                if (sp == SP_LAB || sp == SP_YCRCB) {
-                    for (int k = 0; k < m; ++k) {
-                        const PyrPlan& pp = plans[base + k];
-                        PyrItem& it = B.it[k];
-                        it.src = pyrs[base + k] + pp.img_off[l]; it.sw = pp.W[l]; it.sh = pp.H[l];
-                        it.srow = pp.img_row[l]; it.splane = pp.img_plane[l];
-                        it.dst = pyrs[base + k] + pp.cimg_off[s][l];
-                        it.mode = sp;
-                    }
-                    k_convert<<<grid(mw, mh, m), blk, 0, st>>>(B);
-                }
-                for (int k = 0; k < m; ++k) {
-                    const PyrPlan& pp = plans[base + k];
-                    PyrItem& it = B.it[k];
-                    it.src = pyrs[base + k] + pp.cimg_off[s][l]; it.sw = pp.W[l]; it.sh = pp.H[l];
-                    it.srow = pp.img_row[l]; it.splane = pp.img_plane[l];
-                    it.dst = pyrs[base + k] + pp.desc_off[s][l]; it.drow = pp.desc_row[l];
-                    it.split = reinterpret_cast<uint32_t*>(pyrs[base + k] + pp.split_off[s][l]);
-                }
-                dim3 g((mw + SB_TW - 1) / SB_TW, (mh + SB_TH - 1) / SB_TH, m);
-                const dim3 sblk(SB_TW, SB_TY);
-                if (p->sobel == 5) {
-                    if (C == 1) k_sobel<5, 1><<<g, sblk, 0, st>>>(B, dir_only);
-                    else k_sobel<5, 3><<<g, sblk, 0, st>>>(B, dir_only);
+        // every level and direction of every image, PYR_MAXB items a launch
+        auto items = [&](int what) {              // 0 conversion, 1 gradients, 2 bit-planes
+            int at = 0, launches = 0;
+            auto flush = [&]() {
+                B.n = at;
+                const int blocks = B.cum[at];
+                at = 0;
+                if (blocks == 0) return;
+                ++launches;
+                if (what == 0) {
+                    k_convert<<<blocks, 256, 0, st>>>(B);
+                } else if (what == 2) {
+                    if (C == 3) k_bits<6><<<blocks, dim3(32, 8), 0, st>>>(B);
+                    else k_bits<2><<<blocks, dim3(32, 8), 0, st>>>(B);
                 } else {
-                    if (C == 1) k_sobel<3, 1><<<g, sblk, 0, st>>>(B, dir_only);
-                    else k_sobel<3, 3><<<g, sblk, 0, st>>>(B, dir_only);
+                    const dim3 sblk(SB_TW, SB_TY);
+                    if (p->sobel == 5) {
+                        if (C == 1) k_sobel<5, 1><<<blocks, sblk, 0, st>>>(B, dir_only);
+                        else k_sobel<5, 3><<<blocks, sblk, 0, st>>>(B, dir_only);
+                    } else {
+                        if (C == 1) k_sobel<3, 1><<<blocks, sblk, 0, st>>>(B, dir_only);
+                        else k_sobel<3, 3><<<blocks, sblk, 0, st>>>(B, dir_only);
+                    }
                 }
-                if (dir_only == 1) {                   // the sign codes as bit-planes
-                    int mb = 0;
+            };
+            B.cum[0] = 0;
+            for (int l = 0; l < L; ++l)           // the large levels first
+                for (int s = 0; s < nsch; ++s) {
+                    const int sp = p0.space[s][l];
+                    if (what == 0 && sp != SP_LAB && sp != SP_YCRCB) continue;
                     for (int k = 0; k < m; ++k) {
                         const PyrPlan& pp = plans[base + k];
-                        PyrItem& it = B.it[k];
-                        it.bits = reinterpret_cast<uint32_t*>(pyrs[base + k] + pp.bits_off[s][l]);
-                        it.brow = pp.bit_row[l];
-                        mb = pp.bit_row[l] > mb ? pp.bit_row[l] : mb;
+                        uint8_t* pyr = pyrs[base + k];
+                        PyrItem& it = B.it[at];
+                        it.sw = pp.W[l]; it.sh = pp.H[l];
+                        it.srow = pp.img_row[l]; it.splane = pp.img_plane[l];
+                        int blocks;
+                        if (what == 0) {
+                            it.src = pyr + pp.img_off[l];
+                            it.dst = pyr + pp.cimg_off[s][l];
+                            it.mode = sp;
+                            blocks = ((it.sw + CV_W - 1) / CV_W) * ((it.sh + CV_H - 1) / CV_H);
+                        } else {
+                            it.src = pyr + pp.cimg_off[s][l];
+                            it.dst = pyr + pp.desc_off[s][l]; it.drow = pp.desc_row[l];
+                            it.split = reinterpret_cast<uint32_t*>(pyr + pp.split_off[s][l]);
+                            blocks = ((it.sw + SB_TW - 1) / SB_TW) * ((it.sh + SB_TH - 1) / SB_TH);
+                        }
+                        if (what == 2) {
+                            it.bits = reinterpret_cast<uint32_t*>(pyr + pp.bits_off[s][l]);
+                            it.brow = pp.bit_row[l];
+                            blocks = ((it.brow + 31) / 32) * ((it.sh + 2 * BORD + 7) / 8);
+                        }
+                        B.cum[at + 1] = B.cum[at] + blocks;
+                        if (++at == PYR_MAXB) flush();
                     }
-                    const dim3 gb((mb + 31) / 32, (mh + 2 * BORD + 7) / 8, m);
-                    if (C == 3) k_bits<6><<<gb, dim3(32, 8), 0, st>>>(B);
-                    else k_bits<2><<<gb, dim3(32, 8), 0, st>>>(B);
                 }
-            }
+            flush();
+            return launches;
+        };
+        ks.n = L + items(0) + items(1) + (dir_only == 1 ? items(2) : 0);
         if (pgm_status r = launch_status("pyramid: launch"); r != PGM_OK) return r;
     }
     return PGM_OK;
