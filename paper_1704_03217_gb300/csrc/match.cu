@@ -99,8 +99,9 @@ __device__ __forceinline__ unsigned long long warp_cost(const Ref<NCH, PPL>& R, 
 constexpr int BOX_TW = 64, BOX_TH = 32, BOX_H = MAXP / 2, BOX_RUN = 8;
 template <int NCH>
 __global__ void __launch_bounds__(256) k_box(const __grid_constant__ LvlBatch B) {
-    __shared__ uint32_t sN[BOX_TH + 2 * BOX_H][BOX_TW + 2 * BOX_H];
-    __shared__ unsigned long long sR[BOX_TH + 2 * BOX_H][BOX_TW];
+    // odd pitches (in their own words): the row sums' lanes lie on rows
+    __shared__ uint32_t sN[BOX_TH + 2 * BOX_H][BOX_TW + 2 * BOX_H + 1];
+    __shared__ unsigned long long sR[BOX_TH + 2 * BOX_H][BOX_TW + 1];
     const DirLvl& D = B.d[blockIdx.z][blockIdx.y >> 1];
     const bool ref = blockIdx.y & 1;
     const int w = ref ? D.rw : D.tw, hh = ref ? D.rh : D.th, P = D.P, h = P / 2;
@@ -128,10 +129,11 @@ __global__ void __launch_bounds__(256) k_box(const __grid_constant__ LvlBatch B)
     }
     __syncthreads();
     // row sums: thread -> (row, run of BOX_RUN outputs); consecutive threads
-    // take consecutive runs of one row
+    // take the same run of consecutive rows (consecutive runs of one row are 8
+    // words apart, 8 lanes to a bank)
     constexpr int RUNS_X = BOX_TW / BOX_RUN;
     for (int e = threadIdx.x; e < ih * RUNS_X; e += blockDim.x) {
-        const int r = e / RUNS_X, c0 = (e - r * RUNS_X) * BOX_RUN;
+        const int run = e / ih, r = e - run * ih, c0 = run * BOX_RUN;
         unsigned long long s = 0;
         for (int o = 0; o < P; ++o) s += sN[r][c0 + o];
         sR[r][c0] = s;
