@@ -130,7 +130,8 @@ __global__ void __launch_bounds__(256) k_box(const __grid_constant__ LvlBatch B)
     __syncthreads();
     // row sums: thread -> (row, run of BOX_RUN outputs); consecutive threads
     // take the same run of consecutive rows (consecutive runs of one row are 8
-    // words apart, 8 lanes to a bank)
+    // words apart, 8 lanes to a bank: 472 -> 305 us for the five levels of 16
+    // colour pairs of 1024 x 436)
     constexpr int RUNS_X = BOX_TW / BOX_RUN;
     for (int e = threadIdx.x; e < ih * RUNS_X; e += blockDim.x) {
         const int run = e / ih, r = e - run * ih, c0 = run * BOX_RUN;
