@@ -5,9 +5,13 @@
 // 4-adjacency, two neighbours joining iff |u_s - u_t|^2 < region_dmax2.  They
 // are found with a lock-free union-find whose links always point to the
 // smaller index, so after path compression every seed carries the smallest
-// index of its component whatever the thread order.  Components are then
-// sized with atomics; survivors (size >= min_region) are compacted in lattice
-// raster order by a three-pass scan.
+// index of its component whatever the thread order.  Seeds start linked to the
+// first of their horizontal run within a warp's 32 seeds, and of the vertical
+// pairs between two runs only the leftmost is united.  Components are then
+// sized with atomics, a warp's seeds of one component together (one atomic per
+// seed of a component that spans the image is a queue at one address);
+// survivors (size >= min_region) are compacted in lattice raster order by a
+// three-pass scan.
 #include "pgm_device.cuh"
 
 namespace pgm {
@@ -52,14 +56,27 @@ __device__ void unite(int* L, int a, int b) {
     }
 }
 
+// lattice neighbours a, b (both inside the field) lie in one region
+__device__ __forceinline__ bool joined(const FiltItem& it, int dmax2, int a, int b) {
+    if (!inlier(it.flags[a]) || !inlier(it.flags[b])) return false;
+    const int32_t ua = it.u[a], ub = it.u[b];
+    const long long dx = lo16(ua) - lo16(ub), dy = hi16(ua) - hi16(ub);
+    return dx * dx + dy * dy < dmax2;
+}
+
 // All kernels take a batch of fields: blockIdx.y (blockIdx.x for the scan)
 // selects the pair; blocks past a pair's seed count return.
 __global__ void k_cc_init(const __grid_constant__ FiltBatch F) {
     const FiltItem& it = F.it[blockIdx.y];
     const int n = it.nx * it.ny;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x * (int)blockDim.x >= n) return;          // whole block
+    const bool head = s >= n || lane == 0 || s % it.nx == 0 || !joined(it, F.dmax2, s - 1, s);
+    const unsigned heads = __ballot_sync(0xffffffffu, head);
     if (s >= n) return;
-    it.label[s] = inlier(it.flags[s]) ? s : -1;
+    // the last head at or before this lane
+    const int first = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    it.label[s] = inlier(it.flags[s]) ? s - (lane - first) : -1;
     it.size[s] = 0;
 }
 
@@ -69,28 +86,34 @@ __global__ void k_cc_link(const __grid_constant__ FiltBatch F) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nx * ny || !inlier(it.flags[s])) return;
     const int i = s % nx, j = s / nx;
-    const int32_t us = it.u[s];
-    if (i + 1 < nx && inlier(it.flags[s + 1])) {
-        const int32_t ut = it.u[s + 1];
-        const long long dx = lo16(us) - lo16(ut), dy = hi16(us) - hi16(ut);
-        if (dx * dx + dy * dy < F.dmax2) unite(it.label, s, s + 1);
-    }
-    if (j + 1 < ny && inlier(it.flags[s + nx])) {
-        const int32_t ut = it.u[s + nx];
-        const long long dx = lo16(us) - lo16(ut), dy = hi16(us) - hi16(ut);
-        if (dx * dx + dy * dy < F.dmax2) unite(it.label, s, s + nx);
-    }
+    const bool left = i > 0 && joined(it, F.dmax2, s - 1, s);
+    if (left && (s & 31) == 0) unite(it.label, s, s - 1);        // runs end with a warp
+    // the seed below, unless the pair to the left says the same: that pair is
+    // joined, and so are both of its seeds with these
+    if (j + 1 < ny && joined(it, F.dmax2, s, s + nx) &&
+        !(left && joined(it, F.dmax2, s + nx - 1, s + nx) && joined(it, F.dmax2, s - 1, s + nx - 1)))
+        unite(it.label, s, s + nx);
 }
 
 __global__ void k_cc_flatten(const __grid_constant__ FiltBatch F) {
     const FiltItem& it = F.it[blockIdx.y];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= it.nx * it.ny || it.label[s] < 0) return;
-    // read-only find: a halving store by another thread could otherwise
-    // overwrite the root just written to label[s] with a non-root ancestor
-    const int r = find_root(it.label, s);
-    it.label[s] = r;
-    atomicAdd(&it.size[r], 1);
+    const int n = it.nx * it.ny;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x * (int)blockDim.x >= n) return;          // whole block
+    int r = -1;
+    if (s < n && it.label[s] >= 0) {
+        // read-only find: a halving store by another thread could otherwise
+        // overwrite the root just written to label[s] with a non-root ancestor
+        r = find_root(it.label, s);
+        it.label[s] = r;
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, r >= 0);
+    while (todo) {                                               // (uniform over the warp)
+        const int lead = __ffs(todo) - 1, r0 = __shfl_sync(0xffffffffu, r, lead);
+        const unsigned same = __ballot_sync(0xffffffffu, r == r0);
+        if (lane == lead) atomicAdd(&it.size[r0], __popc(same));
+        todo &= ~same;
+    }
 }
 
 // pass 1: survivors per block of 256 seeds
