@@ -125,6 +125,9 @@ inline pgm_status launch_status(const char* site) {
 // maximum (a launch still uses only what it asks for) and never lowered.
 pgm_status smem_opt_in(const void* kern);
 
+// SMs of the current device (0 on a CUDA error).
+int device_sms();
+
 pgm_status check_params(const pgm_params* p);
 bool make_pyr_plan(const pgm_params* p, int w, int h, PyrPlan* pp);
 bool make_ws_plan(const pgm_params* p, int w1, int h1, int w2, int h2, WsPlan* wp);

@@ -1795,7 +1795,7 @@ static_assert(sizeof(LvlBatch) + sizeof(MatchConst) + sizeof(RowSched) + sizeof(
                   2 * sizeof(int) + sizeof(long long) + 256 <= 32764,
               "k_pm_r parameters exceed the kernel parameter limit");
 
-static int device_sms() {
+int device_sms() {
     static thread_local int dev_cached = -1, sms = 0;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -2041,17 +2041,25 @@ bool pm_tile_fits(const LvlBatch& B, const MatchConst& mc, int nch) {
     return pr_plan(B, mc, nch, S, G);
 }
 
-// Phases larger than one tile per SM run one launch per direction.
+// Tiles per SM up to which both directions share a launch.  The int16 kernels
+// are specialised for a direction's patch side and overlap on two streams: one.
+// The bit-plane kernels do not depend on the patch side, and one launch saves a
+// ramp: at 1 / 12 / 24 tiles one 640 x 480 gray pair takes 619 / 588 / 588 us,
+// four 1024 x 436 colour pairs 1982 / 1940 / 1938, 16 of them 5591 / 5554 / 5553
+// (int16 at 3 / 6 / 12: a colour pair 1154 -> 1159 / 1158 / 1241).
+static int both_limit(const MatchConst& mc) { return (use_bits(mc) ? 24 : 1) * device_sms(); }
+
+// Larger phases run one launch per direction.
 bool pm_tile_split(const LvlBatch& B, const MatchConst& mc, int nch) {
     RowSched S[3];
     RowGeom G[2];
     return pr_plan(B, mc, nch, S, G) && !pm_direct_fits(B, mc, nch, device_sms()) &&
-           (S[2].total > device_sms() || 2 * B.n > PR_MAPS);
+           (S[2].total > both_limit(mc) || 2 * B.n > PR_MAPS);
 }
 
 // *handled = false when pr_plan refuses the batch; the caller then uses the
-// per-seed kernels.  A small phase (at most one tile per SM, the coarse
-// levels) runs both directions in one launch of the run-time-P consumer; a
+// per-seed kernels.  A phase of few seeds goes to pm_direct.cu.  Up to both_limit
+// tiles both directions run in one launch (int16: of the run-time-P consumer); a
 // larger one runs each direction in its own launch of the consumer for its
 // patch side, the backward one on st2 when given (the two directions are
 // independent within a phase).  *nlaunch: kernels launched.
@@ -2070,7 +2078,7 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
         return launch_pm_direct(B, mc, nch, st);
     }
     const bool bits = use_bits(mc);
-    if (S[2].total <= device_sms() && 2 * B.n <= PR_MAPS) {
+    if (S[2].total <= both_limit(mc) && 2 * B.n <= PR_MAPS) {
         const int words = G[0].words > G[1].words ? G[0].words : G[1].words;
         *nlaunch = 1;
         RowMaps& TM = pr_maps(B, nch, bits, S[2], G);
