@@ -76,8 +76,8 @@ namespace {
 
 constexpr int TC_M = 128;              // flattened seeds per tile
 constexpr int TC_N = 160;              // flattened target centres per tile
-constexpr int TC_NT = 2;               // centre tiles per CTA, whole patches staged
-constexpr int TC_NTC = 4;              // centre tiles per CTA, patches staged in chunks
+constexpr int TC_NT = 2;               // centre tiles per CTA, whole patches staged, and
+constexpr int TC_NTC = 4;              // patches staged in chunks; one each for a small grid
 constexpr int TC_WORKERS = 8;          // staging and epilogue warps
 constexpr int TC_THREADS = 32 * (TC_WORKERS + 1);
 constexpr int TC_MAXP = 15;            // the exact-accumulation bound above
@@ -90,7 +90,7 @@ constexpr long long TC_DRAIN_CYCLES = 1ll << 31;
 // The K steps of each direction's patch, chunk after chunk (first step of
 // chunk c: n0[c]); a chunk is Q sigma patch rows.
 struct TcSteps {
-    int nchunk[2], Q[2];
+    int nchunk[2], Q[2], per[2];       // per: centre tiles per CTA
     int n0[2][TC_MAXP + 1];
     uint16_t pr[2][TC_MAXSTEP];        // p1 | r1 << 4 | p2 << 8 | r2 << 12; p2 = 15: zero partner
 };
@@ -102,7 +102,8 @@ struct TcGeom {
 };
 
 // Q: phase rows per chunk, nchunk chunks; gray: the runs' second copy
-__host__ __device__ inline TcGeom tc_geom(const DirLvl& D, int sigma, int Q, int nchunk, bool gray) {
+__host__ __device__ inline TcGeom tc_geom(const DirLvl& D, int sigma, int Q, int nchunk, int per,
+                                          bool gray) {
     TcGeom g;
     const int P = D.P;
     g.e = (P - 1) / sigma;
@@ -113,13 +114,12 @@ __host__ __device__ inline TcGeom tc_geom(const DirLvl& D, int sigma, int Q, int
     g.pa = g.Wu < ra ? g.Wu : ra;
     g.LA = g.pa * (Q - 1) + ra;
     g.copies = gray && P % 4 ? 2 : 1;
-    g.NT = nchunk > 1 ? 1 : TC_NT;                     // tiles staged together
+    g.NT = nchunk > 1 ? 1 : per;                       // tiles staged together
     g.Wt = D.tw + P - 1;
     g.ntiles = (D.th * g.Wt + TC_N - 1) / TC_N;
     const int rb = g.NT * TC_N + P - 1, rows = Q * sigma < P ? Q * sigma : P;
     g.pb = g.Wt < rb ? g.Wt : rb;
     g.LB = g.pb * (rows - 1) + rb;
-    const int per = nchunk > 1 ? TC_NTC : TC_NT;
     g.bands = (g.ntiles + per - 1) / per;
     g.ctas = g.mtiles * g.bands;
     g.bufs = nchunk > 1 ? 2 : 1;
@@ -262,10 +262,11 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
     const DirLvl& D = B.d[pair][dir];
     const int sg = mc.sigma, P = D.P, h = P / 2;
     const int nchunk = T.nchunk[dir], Q = T.Q[dir];
-    const TcGeom g = tc_geom(D, sg, Q, nchunk, GRAY);
+    const int per = T.per[dir];
+    const TcGeom g = tc_geom(D, sg, Q, nchunk, per, GRAY);
     if ((int)blockIdx.x >= g.ctas || D.nx * D.ny == 0) return;
     const int mt = blockIdx.x % g.mtiles, band = blockIdx.x / g.mtiles;
-    const int m0 = mt * TC_M, per = nchunk > 1 ? TC_NTC : TC_NT;
+    const int m0 = mt * TC_M;
     const int tile0 = band * per, ntile = min(per, g.ntiles - tile0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tail = 4 * ((P - 1) / 4);                // first column of a gray row's last run
@@ -600,23 +601,33 @@ pgm_status launch_init_tc(const LvlBatch& B, const MatchConst& mc, int nch, bool
             if (D.P < 1 || D.P > TC_MAXP || D.P != P) return PGM_OK;
             if ((long long)D.tw * D.th >= (1ll << 24) || !D.sa2img || !D.sb2) return PGM_OK;
         }
-        // the fewest chunks whose staging fits for every pair of the batch
+        // the fewest chunks whose staging fits for every pair of the batch, and
+        // one centre tile a CTA where more would leave SMs without one (a
+        // 1024 x 436 pair had 28 CTAs with two tiles each: 1150 -> 1121 us a call,
+        // a 256 x 192 gray one 474 -> 465; no gain with the line at two or four
+        // CTAs a SM)
         const int nq = (P - 1) / mc.sigma + 1;
-        int Q = 0, nchunk = 0, most = 0, grid = 0;
+        int Q = 0, nchunk = 0, most = 0, grid = 0, per = 0;
         for (int want = 1; want <= nq && nchunk == 0; ++want) {
             Q = (nq + want - 1) / want;
             const int nc = (nq + Q - 1) / Q;
-            most = grid = 0;
-            for (int k = 0; k < B.n; ++k) {
-                const TcGeom g = tc_geom(B.d[k][d], mc.sigma, Q, nc, gray);
-                most = std::max(most, tc_units(g));
-                grid = std::max(grid, g.ctas);
+            for (per = nc > 1 ? TC_NTC : TC_NT;; per = 1) {
+                int all = 0;
+                most = grid = 0;
+                for (int k = 0; k < B.n; ++k) {
+                    const TcGeom g = tc_geom(B.d[k][d], mc.sigma, Q, nc, per, gray);
+                    most = std::max(most, tc_units(g));
+                    grid = std::max(grid, g.ctas);
+                    all += g.ctas;
+                }
+                if (per == 1 || 2 * all > device_sms()) break;     // (two directions)
             }
             if (16L * most <= TC_SMEM) nchunk = nc;
         }
         if (nchunk == 0) return PGM_OK;
         T.nchunk[d] = nchunk;
         T.Q[d] = Q;
+        T.per[d] = per;
         int n = 0;
         for (int c = 0; c < nchunk; ++c) {
             T.n0[d][c] = n;
