@@ -13,7 +13,9 @@
 // of 2 x 4, 1 x 4, 1 x 8), each target word
 // loaded once for all seeds and each reference word (a broadcast) once for
 // all centres.  A patch row is summed in 32 bits (at most 48 words: below
-// 2^31 for any descriptor value), the rows in 64 bits.
+// 2^31 for any descriptor value), the rows in 64 bits.  It takes what the tensor
+// cores' form (init_tc.cu) refuses, patches of 16 and strides above 5, where the
+// target image fits.
 #include "match_common.cuh"
 
 namespace pgm {

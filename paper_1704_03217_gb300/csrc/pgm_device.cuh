@@ -278,8 +278,8 @@ pgm_status launch_box(const LvlBatch& B, int nch, int max_pixels, cudaStream_t s
 // (*nlaunch: the kernels launched)
 pgm_status launch_init_tile(const LvlBatch& B, const MatchConst& mc, int nch, bool* handled,
                             cudaStream_t st, int* nlaunch);
-// init_tc.cu: the same initialisation on the tensor cores (six channels,
-// squared L2, patches up to 15 x 15); *handled = false when it does not apply
+// init_tc.cu: the same initialisation on the tensor cores (squared L2, patches
+// up to 15 x 15); *handled = false when it does not apply
 pgm_status launch_init_tc(const LvlBatch& B, const MatchConst& mc, int nch, bool* handled,
                           cudaStream_t st, int* nlaunch);
 // true when the tile search kernel takes this batch (it then also does the
