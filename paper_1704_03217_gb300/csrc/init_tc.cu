@@ -163,10 +163,6 @@ __device__ __forceinline__ bool tc_mbar_wait(uint32_t bar, uint32_t parity, long
 __device__ __forceinline__ void tc_mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-// the worker warps only
-__device__ __forceinline__ void tc_worker_sync() {
-    asm volatile("bar.sync 1, %0;\n" ::"n"(32 * TC_WORKERS) : "memory");
-}
 __device__ __forceinline__ void tc_fence_before() {
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
 }
@@ -277,7 +273,8 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
     uint4* sBuf = sS + TC_MAXSTEP;
     uint4* sZ = sBuf + g.bufs * g.buf_units;           // TC_N zero rows
     unsigned long long* sBest = reinterpret_cast<unsigned long long*>(sZ + TC_N);   // [2][TC_M]
-    const uint32_t bar_full = smem_u32(sm4), bar_done = bar_full + 16, bar_acc = bar_full + 32;
+    const uint32_t bar_full = smem_u32(sm4), bar_done = bar_full + 16, bar_acc = bar_full + 32,
+                   bar_tab = bar_full + 48;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm4) + 10;
     volatile int* s_abort = reinterpret_cast<volatile int*>(sm4) + 11;
     const int hl_a = g.copies * g.phases * g.LA;       // units from the high to the low parts
@@ -289,6 +286,7 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
             tc_mbar_init(bar_done + 8 * b, 1);
         }
         tc_mbar_init(bar_acc, TC_WORKERS);
+        tc_mbar_init(bar_tab, TC_WORKERS);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -425,8 +423,13 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
         unsigned long long best = INF;
         bool ok = true;
         // centres of a tile's columns: sum |b|^2 (INF: not a centre) and raster
-        // index; two tables in turn, each written before a wait that every
-        // worker warp passes and read after it
+        // index; two tables in turn.  A worker warp arrives on bar_tab once it
+        // has written its part of tile k's table and read the whole of tile
+        // k - 1's, and waits for that phase before it reads tile k's table or
+        // writes tile k + 1's.  Every wait between the workers is such a
+        // bounded one: a warp whose wait runs out leaves for the __syncthreads
+        // at the end, and the others, which it may have left behind at any
+        // point, must not wait for it without a limit.
         auto centres = [&](int k) {
             for (int j = wt; j < TC_N; j += WT) {
                 const int n = (tile0 + k) * TC_N + j, y = n / g.Wt, x = n - y * g.Wt;
@@ -435,6 +438,9 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
                 sQ[(k & 1) * TC_N + j] =
                     make_uint4((uint32_t)sb, (uint32_t)(sb >> 32), (uint32_t)(y * D.tw + x), 0u);
             }
+        };
+        auto tables = [&](int k) {
+            return __all_sync(FULL, tc_mbar_wait(bar_tab, (uint32_t)k & 1u, limit, s_abort)) != 0;
         };
         // the accumulators of tile k, complete once `waits` commits are on buffer b
         auto finish = [&](int k, int b, int waits) {
@@ -468,13 +474,13 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
         if (nchunk == 1) {
             for (int k = 0; k < ntile; ++k) centres(k);
             stage(tile0, 0, 0);
-            for (int k = 0; k < ntile && ok; ++k) {
-                if (k == 0) tc_worker_sync();          // the centre tables
-                ok = finish(k, 0, k);
-            }
+            if (lane == 0) tc_mbar_arrive(bar_tab);
+            ok = tables(0);
+            for (int k = 0; k < ntile && ok; ++k) ok = finish(k, 0, k);
         } else {
             for (int i = 0; i <= nstage && ok; ++i) {
                 const int b = i & 1, k = i / nchunk, c = i - k * nchunk;
+                if (i > 0 && c == 0 && !(ok = tables(k - 1))) break;
                 if (i < nstage) {
                     // the MMAs of the buffer's last chunk are done
                     if (i >= 2)
@@ -484,10 +490,9 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
                     if (c == 0) centres(k);
                     stage(tile0 + k, c, b);
                 }
-                if (i > 0 && c == 0) {                 // the tile before is complete
-                    tc_worker_sync();
+                if (i > 0 && c == 0)                   // the tile before is complete
                     ok = finish(k - 1, b ^ 1, (i - 1) / 2);
-                }
+                if (c == 0 && ok && i < nstage && lane == 0) tc_mbar_arrive(bar_tab);
             }
         }
         if (!ok) {
