@@ -321,13 +321,14 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
     // of every tile; tiles are finished in order either way
     const int nstage = nchunk > 1 ? ntile * nchunk : 1;
 
+    int issued[2] = {0, 0};                            // (issuing thread) commits so far on each
+                                                       // buffer's barrier
     if (warp == TC_WORKERS) {
         // ------------------------------------------------ MMA issue (one thread)
         if (lane == 0) {
             const uint32_t idesc = (1u << 4) | ((uint32_t)(TC_N >> 3) << 17) |
                                    ((uint32_t)(TC_M >> 4) << 24);   // M 128, N 160, fp16 K-major, fp32
             const uint32_t aZ = smem_u32(sZ);
-            int issued[2] = {0, 0};                    // commits so far on each buffer's barrier
             bool ok = true;
             for (int k = 0; k < ntile && ok; ++k) {
                 // the previous tile's accumulators have been read
@@ -363,10 +364,6 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
             if (!ok) {
                 if (!*s_abort) atomicOr(B.err[pair], (unsigned)PGM_ERR_TIMEOUT);
                 *s_abort = 1;
-                for (int b = 0; b < 2; ++b)            // let the issued MMAs finish
-                    if (issued[b])
-                        (void)tc_mbar_wait(bar_done + 8 * b, (uint32_t)(issued[b] - 1) & 1u,
-                                           TC_DRAIN_CYCLES, nullptr);
             }
         }
         __syncwarp();
@@ -511,6 +508,14 @@ k_init_tc(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_
         const int mm = m0 + tid, i = mm % g.Wu, j = mm / g.Wu;
         if (i < D.nx && j < D.ny && bb != INF) atomicMin(D.cost + (size_t)j * D.nx + i, bb);
     }
+    // whichever warp gave up: the issued MMAs read shared memory and write tensor
+    // memory until they finish (the last commit on each buffer is the only one
+    // that can be outstanding; without an abort every one has been waited for)
+    if (*s_abort && warp == TC_WORKERS && lane == 0)
+        for (int b = 0; b < 2; ++b)
+            if (issued[b])
+                (void)tc_mbar_wait(bar_done + 8 * b, (uint32_t)(issued[b] - 1) & 1u, TC_DRAIN_CYCLES,
+                                   nullptr);
     tc_fence_before();
     __syncthreads();
     if (warp == TC_WORKERS) {

@@ -4,7 +4,8 @@ accumulators, one issuing thread, and the tensor pipe that completes its
 commits at some later time.  Every bounded wait may run out at any moment, as
 it may on the GPU, where the lanes of a warp look at the barrier, the abort
 flag and the clock one after another.  All interleavings of two workers are
-walked: each ends with every warp at the block's last barrier; no wait passes
+walked: each ends with every warp at the block's last barrier, behind which no
+product is in flight when the tensor memory is freed; no wait passes
 on a phase that it does not mean; a centre table is read complete and not
 written meanwhile; a buffer is not staged again under the products that read
 it; and accumulators are neither read before their products
@@ -47,7 +48,10 @@ def worker(nchunk, ntile, meet):
     return ops + [("join",)]
 
 
-def issuer(nchunk, ntile):
+def issuer(nchunk, ntile, drain):
+    """drain: who waits for the products in flight after an abort: "joined",
+    the issuer behind the block's barrier, or "own", the issuer when its own
+    wait ran out."""
     ops = []
     for k in range(ntile):
         if k:
@@ -57,17 +61,17 @@ def issuer(nchunk, ntile):
             b = i & 1 if nchunk > 1 else 0
             if nchunk > 1 or k == 0:
                 ops.append(("wait", "full%d" % b, i // 2))
-            ops.append(("issue", k, b, c == nchunk - 1))
-    return ops + [("join",)]
+            ops.append(("issue", k, b))
+    return ops + ([("drain",)] if drain == "own" else []) + [("join",)]
 
 
 BARS = ("full0", "full1", "done0", "done1", "acc", "tab")
 
 
-def walk(nchunk, ntile, meet, failing, workers=2):
+def walk(nchunk, ntile, meet, failing, drain="joined", workers=2):
     """Every interleaving; a violation message or None.  failing: waits may
     run out."""
-    progs = [worker(nchunk, ntile, meet)] * workers + [issuer(nchunk, ntile)]
+    progs = [worker(nchunk, ntile, meet)] * workers + [issuer(nchunk, ntile, drain)]
     count = {b: 1 if b.startswith("done") else workers for b in BARS}
     # program counters; barriers (phase, arrived); abort; commits in flight
     # (tile, buffer); tiles of both tables' parts per worker; workers that
@@ -106,7 +110,10 @@ def walk(nchunk, ntile, meet, failing, workers=2):
                         return "wait for phase %d of %s passed in phase %d" % (op[2], op[1], ph)
                     step(a, pc + 1)
                 if failing:                                # (abort seen, or out of time)
-                    step(a, len(prog) - 1, abort=True)
+                    step(a, len(prog) - (2 if prog[-2] == ("drain",) else 1), abort=True)
+            elif op[0] == "drain":
+                if not flight:
+                    step(a, pc + 1)
             elif op[0] == "arrive":
                 if op[1].startswith("full") and nchunk > 1 and done < 2 * op[2] + int(op[1][4]) - 1:
                     return "buffer %s restaged under its products" % op[1][4]
@@ -132,7 +139,12 @@ def walk(nchunk, ntile, meet, failing, workers=2):
                 k = op[1]
                 if k and reads[k - 1] < workers:
                     return "accumulators of tile %d overwritten before they were read" % (k - 1)
-                step(a, pc + 1, flight=flight + ((k, op[2]),))
+                step(a, pc + (2 if prog[pc + 1] == ("drain",) else 1), flight=flight + ((k, op[2]),))
+        if flight and all(progs[a][pcs[a]] == ("join",) for a in range(workers + 1)):
+            if drain == "own" or not abort:
+                return "tensor memory freed under %d commits" % len(flight)
+            if len({b for _, b in flight}) < len(flight):
+                return "two commits outstanding on one buffer"
         if not out:
             if any(progs[a][pcs[a]] != ("join",) for a in range(workers + 1)):
                 return "stuck at %s" % [progs[a][pcs[a]] for a in range(workers + 1)]
@@ -164,6 +176,13 @@ def test_a_barrier_without_a_limit_strands_a_worker(nchunk, ntile):
     a wait that ran out, another passes it and waits for the first for ever."""
     assert walk(nchunk, ntile, "named", False) is None
     assert "stuck" in walk(nchunk, ntile, "named", True)
+
+
+@pytest.mark.parametrize("nchunk,ntile", [(1, 1), (1, 2), (2, 2), (3, 1)])
+def test_a_drain_on_the_issuers_own_failure_alone_is_not_enough(nchunk, ntile):
+    """A worker's wait runs out after the issuer has issued everything."""
+    assert walk(nchunk, ntile, "mbarrier", False, drain="own") is None
+    assert "freed" in walk(nchunk, ntile, "mbarrier", True, drain="own")
 
 
 def test_the_kernel_has_no_other_unbounded_barrier():
