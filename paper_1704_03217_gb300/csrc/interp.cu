@@ -374,11 +374,15 @@ pgm_status pgm_interpolate(const pgm_params* p, const void* d_pyr1, int w, int h
     }
     // relax until a launch changes nothing, in groups of launches between two
     // looks at their flags (a launch after one that changed nothing returns at
-    // once); a bound far above any path length in tiles keeps a defect from
-    // looping for ever.  1024 x 436, k = 16, LA: the call 12.1 -> 3.0 ms
-    // (relaxation 11.6 -> 2.5 in 16 launches, interpolation 1.0 -> 0.47).
+    // once).  The bound keeps a defect from looping for ever: a launch carries
+    // the entries at least one pixel further on their shortest paths (IT_INNER
+    // pixels inside a tile, one where a path crosses between two tiles at every
+    // step; one launch more where a neighbour's list was being written while it
+    // was read), and a path has at most w h pixels.  1024 x 436, k = 16, LA: the
+    // call 12.1 -> 3.0 ms (relaxation 11.6 -> 2.5 in 16 launches, interpolation
+    // 1.0 -> 0.47).
     const dim3 grid(pl.tx, pl.ty);
-    const long long most = 4ll * (long long)w * h / (IT_W * IT_W) + 64;
+    const long long most = 4ll * (long long)w * h + 64;
     long long launches = 0;
     for (bool more = true; more;) {
         if (launches > most) return PGM_ERR_UNSUPPORTED;
