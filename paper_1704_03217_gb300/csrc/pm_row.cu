@@ -461,9 +461,10 @@ __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSch
         // takes 4500 cycles for those; 9.43 -> 9.22 ms a colour step of 16
         // pairs of 1024 x 436, 7.95 -> 7.54 ms a gray one).  With one
         // empty barrier per buffer the tiles are staged in their order (the
-        // warp of tile n - 1 hands on the turn): a warp that looked at a
-        // buffer two tiles ahead would take the parity of the phase before
-        // for its own.
+        // warp of tile n - 1 hands on the turn): in a ring of fewer buffers
+        // than producer warps (the bit-planes' under a wide search window) a
+        // warp could come to a buffer whose last tile but one is not yet
+        // released, and the parity of that phase is the one it waits for.
         if (NG == 0 && n > 0) {
             const unsigned par = (unsigned)(n / NPROD - (pw == 0)) & 1u;
             if (!__all_sync(FULL, mbar_wait(turn0 + 8u * (unsigned)pw, par, limit, abort))) {
