@@ -462,7 +462,7 @@ __device__ void pr_produce(const LvlBatch& B, const MatchConst& mc, const RowSch
         // pairs of 1024 x 436, 7.95 -> 7.54 ms a gray one).  With one
         // empty barrier per buffer the tiles are staged in their order (the
         // warp of tile n - 1 hands on the turn): in a ring of fewer buffers
-        // than producer warps (the bit-planes' under a wide search window) a
+        // than producer warps (the bit-planes' at strides of about 16 and more) a
         // warp could come to a buffer whose last tile but one is not yet
         // released, and the parity of that phase is the one it waits for.
         if (NG == 0 && n > 0) {
