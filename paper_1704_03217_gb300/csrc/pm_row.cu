@@ -1135,18 +1135,16 @@ __device__ __forceinline__ int pg_tile(const LvlBatch& B, const MatchConst& mc, 
     return i - PR_NACT / 2;
 }
 
-// Consumer warps: every tile of the CTA in turn.  PF, PB > 0: the patch side
-// of the forward and the backward tiles (compile time), else at most MAXP
-// (run time).
-template <int PF, int PB>
+// Consumer warps: every tile of the CTA in turn.  PC > 0: the patch side of the
+// launch's direction (compile time), else at most MAXP (run time).
+template <int PC>
 __device__ void pg_consume(const LvlBatch& B, const MatchConst& mc, const RowSched& S,
                            int buf_words, int nbuf, unsigned a_sm, unsigned a_rec,
                            const RowHdr* hdr, const RowGeom* geom, unsigned full0,
                            unsigned empty0, volatile int* abort, long long limit, int warp,
                            int lane, EvCount& ev) {
-    constexpr int NC = pr_cons(2, PF);
-    GrayLane<PF> lf;
-    GrayLane<PB> lb;
+    constexpr int NC = pr_cons(2, PC);
+    GrayLane<PC> L;
     int cur_dir = -1, i0 = warp;
     for (int n = 0;; ++n) {
         const int t = blockIdx.x + n * gridDim.x;
@@ -1162,21 +1160,16 @@ __device__ void pg_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
         const RowHdr H = hdr[b];
         const unsigned buf = a_sm + 4u * (unsigned)(b * buf_words);
         const unsigned rec = a_rec + (unsigned)(sizeof(RowSeed) * PR_NACT) * (unsigned)b;
-        if (PF == PB || H.dir == 0) {
-            if (PF != PB || PF == 0 ? H.dir != cur_dir : cur_dir < 0) lf.set(geom[H.dir], lane & 15);
-            i0 = pg_tile<PF, NC>(B, mc, geom[H.dir], H, lf, buf, rec, i0, lane, ev);
-        } else if constexpr (PF != PB) {
-            if (H.dir != cur_dir) lb.set(geom[H.dir], lane & 15);
-            i0 = pg_tile<PB, NC>(B, mc, geom[H.dir], H, lb, buf, rec, i0, lane, ev);
-        }
+        if (cur_dir < 0) L.set(geom[H.dir], lane & 15);      // (one direction a launch)
         cur_dir = H.dir;
+        i0 = pg_tile<PC, NC>(B, mc, geom[H.dir], H, L, buf, rec, i0, lane, ev);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + 8u * b);         // this warp is done with the buffer
     }
 }
 
-template <int PF, int PB>
-__global__ void __launch_bounds__(32 * (PR_PROD + pr_cons(2, PF)), 1)
+template <int PC>
+__global__ void __launch_bounds__(32 * (PR_PROD + pr_cons(2, PC)), 1)
 k_pm_g(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_constant__ RowSched S,
        const __grid_constant__ RowMaps TM, const int buf_words, const int nbuf,
        const long long limit) {
@@ -1201,7 +1194,7 @@ k_pm_g(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     if (threadIdx.x == 0) {
         for (int b = 0; b < nbuf; ++b) {
             mbar_init(full0 + 8u * b, 1);
-            mbar_init(empty0 + 8u * b, pr_cons(2, PF));
+            mbar_init(empty0 + 8u * b, pr_cons(2, PC));
         }
         for (int p = 0; p < PR_PROD; ++p) mbar_init(turn0 + 8u * p, 1);
         s_abort = 0;
@@ -1210,13 +1203,13 @@ k_pm_g(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
     __syncthreads();
     pdl_wait();                     // the previous phase is complete and visible
     volatile int* abort = &s_abort;
-    if (warp >= pr_cons(2, PF))
+    if (warp >= pr_cons(2, PC))
         pr_produce<2, false, PR_PROD, PR_NBUF>(B, mc, S, TM, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom, full0,
-                        empty0, turn0, abort, limit, warp - pr_cons(2, PF), lane);
+                        empty0, turn0, abort, limit, warp - pr_cons(2, PC), lane);
     else
-        pg_consume<PF, PB>(B, mc, S, buf_words, nbuf, a_sm,
-                                (unsigned)__cvta_generic_to_shared(&s_rec[0][0]), s_hdr, s_geom,
-                                full0, empty0, abort, limit, warp, lane, s_ev);
+        pg_consume<PC>(B, mc, S, buf_words, nbuf, a_sm,
+                       (unsigned)__cvta_generic_to_shared(&s_rec[0][0]), s_hdr, s_geom, full0, empty0,
+                       abort, limit, warp, lane, s_ev);
     ev_flush(s_ev, B);
 }
 
@@ -1231,7 +1224,7 @@ k_pm_g(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
 // it keeps the row's reference bits in registers (NR words per plane) and
 // reads the candidate row as NW staged words per plane, aligned by funnel
 // shifts.  The cost of a candidate is the half-warp sum; costs fit 32 bits.
-template <int NCH, int PC>
+template <int NCH>
 __device__ void pr_consume_bits(const LvlBatch& B, const MatchConst& mc, const RowSched& S,
                                 int buf_words, int nbuf, unsigned a_sm, RowRec (*rec)[PR_NACT],
                                 const RowHdr* hdr, int* next, const RowGeom* geom, unsigned full0,
@@ -1255,7 +1248,7 @@ __device__ void pr_consume_bits(const LvlBatch& B, const MatchConst& mc, const R
         const RowHdr H = hdr[b];
         const RowGeom& G = geom[H.dir];
         const DirLvl& D = B.d[H.pair][H.dir];
-        const int P = PC > 0 ? PC : G.P, h = P / 2;
+        const int P = G.P, h = P / 2;
         const bool live = r < P;
         const int rr = live ? r : 0;
         unsigned msk[NR];                             // the row's bits in each aligned word
@@ -1438,7 +1431,7 @@ __device__ void pr_consume_bits(const LvlBatch& B, const MatchConst& mc, const R
 // deeper ring of staged tiles
 constexpr int PB_PROD = 4, PB_CONS = 20, PB_NBUF = 8;
 
-template <int NCH, int PC>
+template <int NCH>
 __global__ void __launch_bounds__(32 * (PB_PROD + PB_CONS), 1)
 k_pm_b(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_constant__ RowSched S,
        const __grid_constant__ RowMaps TM, const int buf_words, const int nbuf,
@@ -1478,7 +1471,7 @@ k_pm_b(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
                                                 s_next, s_geom, full0, empty0, turn0, abort, limit,
                                                 warp - PB_CONS, lane);
     else
-        pr_consume_bits<NCH, PC>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom,
+        pr_consume_bits<NCH>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_next, s_geom,
                                  full0, empty0, abort, limit, lane, s_ev);
     ev_flush(s_ev, B);
 }
@@ -1598,7 +1591,7 @@ __device__ __forceinline__ void ps_rows(const RowGeom& G, const RowHdr& H, const
     }
 }
 
-template <int NCH, int PC>
+template <int NCH>
 __device__ void ps_consume(const LvlBatch& B, const MatchConst& mc, const RowSched& S, int buf_words,
                            int nbuf, unsigned a_sm, RowRec (*rec)[PR_NACT], const RowHdr* hdr,
                            const RowGeom* geom, unsigned full0, unsigned empty0,
@@ -1623,7 +1616,7 @@ __device__ void ps_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
         const RowHdr H = hdr[b];
         const RowGeom& G = geom[H.dir];
         const DirLvl& D = B.d[H.pair][H.dir];
-        const int P = PC > 0 ? PC : G.P, h = P / 2;
+        const int P = G.P, h = P / 2;
         const unsigned buf = a_sm + 4u * (unsigned)(b * buf_words);
         const unsigned a_rn = buf, a_rs = buf + 4u * (unsigned)G.off_rs;
         const unsigned a_wn = buf + 4u * (unsigned)G.off_win, a_ws = buf + 4u * (unsigned)G.off_ws;
@@ -1745,7 +1738,7 @@ __device__ void ps_consume(const LvlBatch& B, const MatchConst& mc, const RowSch
     }
 }
 
-template <int NCH, int PC>
+template <int NCH>
 __global__ void __launch_bounds__(32 * (PS_PROD + PS_CONS), 1)
 k_pm_s(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_constant__ RowSched S,
        const __grid_constant__ RowMaps TM, const int buf_words, const int nbuf,
@@ -1783,7 +1776,7 @@ k_pm_s(const __grid_constant__ LvlBatch B, const MatchConst mc, const __grid_con
                                                 s_next, s_geom, full0, empty0, 0u, abort, limit,
                                                 warp - PS_CONS, lane);
     else
-        ps_consume<NCH, PC>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_geom, full0, empty0,
+        ps_consume<NCH>(B, mc, S, buf_words, nbuf, a_sm, s_rec, s_hdr, s_geom, full0, empty0,
                             abort, limit, warp, lane, s_ev);
     ev_flush(s_ev, B);
 }
@@ -1968,9 +1961,9 @@ static RowMaps& pr_maps(const LvlBatch& B, int nch, bool bits, const RowSched& S
 // wait limit of the kernel's mbarrier waits (cycles); set by pgm_set_wait_limit
 long long wait_limit();
 
-// Colour (NCH = 6): one direction of patch side PF, staged row pitch PB (0: run
-// time); gray: patch sides of both directions; bit-planes: PF = PB = 0.
-template <int NCH, int PF, int PB, bool BITS = false>
+// int16: one direction of patch side PC (0: run time), colour: staged row pitch
+// SP (0: run time); bit-planes: PC = SP = 0.
+template <int NCH, int PC, int SP = 0, bool BITS = false>
 pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, const RowMaps& TM,
                     int buf_words, cudaStream_t st) {
     const int sms = device_sms();
@@ -1979,9 +1972,9 @@ pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, 
     // tiles of its own, else the warp-per-seed form (coarse levels)
     const bool per_lane = BITS && S.total >= PS_CONS * sms;
     void (*kern)(LvlBatch, MatchConst, RowSched, RowMaps, int, int, long long);
-    if constexpr (BITS) kern = per_lane ? k_pm_s<NCH, 0> : k_pm_b<NCH, 0>;
-    else if constexpr (NCH == 2) kern = k_pm_g<PF, PB>;
-    else kern = k_pm_r<NCH, PF, PB>;
+    if constexpr (BITS) kern = per_lane ? k_pm_s<NCH> : k_pm_b<NCH>;
+    else if constexpr (NCH == 2) kern = k_pm_g<PC>;
+    else kern = k_pm_r<NCH, PC, SP>;
     if (pgm_status r = smem_opt_in((const void*)kern); r != PGM_OK) return r;
     // the ring: as many buffers as fit beside the kernel's static shared
     // memory (the bit-plane kernel's tile records take about 33 KB)
@@ -1995,7 +1988,7 @@ pgm_status launch_r(const LvlBatch& B, const MatchConst& mc, const RowSched& S, 
     while (nbuf < most && (nbuf + 1L) * buf_words * 4 <= cap) ++nbuf;
     const int smem = nbuf * buf_words * 4;
     const int grid = S.total < sms ? S.total : sms;       // one CTA per SM (shared memory)
-    const int threads = !BITS ? 32 * (PR_PROD + pr_cons(NCH, PF))
+    const int threads = !BITS ? 32 * (PR_PROD + pr_cons(NCH, PC))
                         : per_lane ? 32 * (PS_PROD + PS_CONS) : 32 * (PB_PROD + PB_CONS);
     PGM_TRY(launch_pdl(kern, dim3(grid), dim3(threads), smem, st, B, mc, S, TM, buf_words, nbuf,
                        wait_limit()),
@@ -2015,25 +2008,15 @@ pgm_status launch_dir(const LvlBatch& B, const MatchConst& mc, const RowSched& S
             G.off_sb - G.off_win >= G.sp * G.win_h && G.words - G.off_sb >= G.sp + 4 * (P + 2) &&
             G.sp / 4 >= G.win_w + 2)
             return launch_r<6, 15, PR_ROWS_SP>(B, mc, S, TM, buf_words, st);
-        if (P == 15) return launch_r<6, 15, 0>(B, mc, S, TM, buf_words, st);
-        if (P == 11) return launch_r<6, 11, 0>(B, mc, S, TM, buf_words, st);
-        return launch_r<6, 0, 0>(B, mc, S, TM, buf_words, st);
+        if (P == 15) return launch_r<6, 15>(B, mc, S, TM, buf_words, st);
+        if (P == 11) return launch_r<6, 11>(B, mc, S, TM, buf_words, st);
+        return launch_r<6, 0>(B, mc, S, TM, buf_words, st);
     } else {
-        if (P == 15) return launch_r<2, 15, 15>(B, mc, S, TM, buf_words, st);
-        if (P == 11) return launch_r<2, 11, 11>(B, mc, S, TM, buf_words, st);
-        if (P == 8) return launch_r<2, 8, 8>(B, mc, S, TM, buf_words, st);
-        return launch_r<2, 0, 0>(B, mc, S, TM, buf_words, st);
+        if (P == 15) return launch_r<2, 15>(B, mc, S, TM, buf_words, st);
+        if (P == 11) return launch_r<2, 11>(B, mc, S, TM, buf_words, st);
+        if (P == 8) return launch_r<2, 8>(B, mc, S, TM, buf_words, st);
+        return launch_r<2, 0>(B, mc, S, TM, buf_words, st);
     }
-}
-
-// Both directions in one launch.
-template <int NCH>
-pgm_status launch_both(const LvlBatch& B, const MatchConst& mc, const RowSched& S, const RowGeom* G,
-                       const RowMaps& TM, int buf_words, cudaStream_t st) {
-    if constexpr (NCH == 2) {
-        if (G[0].P == G[1].P) return launch_dir<2>(B, mc, S, G[0], TM, buf_words, st);
-    }
-    return launch_r<NCH, 0, 0>(B, mc, S, TM, buf_words, st);
 }
 
 bool pm_tile_fits(const LvlBatch& B, const MatchConst& mc, int nch) {
@@ -2042,28 +2025,29 @@ bool pm_tile_fits(const LvlBatch& B, const MatchConst& mc, int nch) {
     return pr_plan(B, mc, nch, S, G);
 }
 
-// Tiles per SM up to which both directions share a launch.  The int16 kernels
-// are specialised for a direction's patch side and overlap on two streams: one.
-// The bit-plane kernels do not depend on the patch side, and one launch saves a
-// ramp: at 1 / 12 / 24 tiles one 640 x 480 gray pair takes 619 / 588 / 588 us,
-// four 1024 x 436 colour pairs 1982 / 1940 / 1938, 16 of them 5591 / 5554 / 5553
-// (int16 at 3 / 6 / 12: a colour pair 1154 -> 1159 / 1158 / 1241).
-static int both_limit(const MatchConst& mc) { return (use_bits(mc) ? 24 : 1) * device_sms(); }
+// Whether both directions share a launch.  The int16 kernels are specialised for
+// a direction's patch side and overlap on two streams: one launch each (sharing
+// one up to 3 / 6 / 12 tiles per SM: a colour pair 1154 -> 1159 / 1158 / 1241 us;
+// phases of a tile per SM or less go to pm_direct.cu).  The bit-plane kernels do
+// not depend on the patch side, and one launch saves a ramp: up to 24 tiles per
+// SM.  At 1 / 12 / 24 one 640 x 480 gray pair takes 619 / 588 / 588 us, four
+// 1024 x 436 colour pairs 1982 / 1940 / 1938, 16 of them 5591 / 5554 / 5553.
+static bool one_launch(const LvlBatch& B, const MatchConst& mc, const RowSched& both) {
+    return use_bits(mc) && both.total <= 24 * device_sms() && 2 * B.n <= PR_MAPS;
+}
 
-// Larger phases run one launch per direction.
 bool pm_tile_split(const LvlBatch& B, const MatchConst& mc, int nch) {
     RowSched S[3];
     RowGeom G[2];
     return pr_plan(B, mc, nch, S, G) && !pm_direct_fits(B, mc, nch, device_sms()) &&
-           (S[2].total > both_limit(mc) || 2 * B.n > PR_MAPS);
+           !one_launch(B, mc, S[2]);
 }
 
 // *handled = false when pr_plan refuses the batch; the caller then uses the
-// per-seed kernels.  A phase of few seeds goes to pm_direct.cu.  Up to both_limit
-// tiles both directions run in one launch (int16: of the run-time-P consumer); a
-// larger one runs each direction in its own launch of the consumer for its
-// patch side, the backward one on st2 when given (the two directions are
-// independent within a phase).  *nlaunch: kernels launched.
+// per-seed kernels.  A phase of few seeds goes to pm_direct.cu.  Else both
+// directions run in one launch (one_launch), or each in its own launch of the
+// consumer for its patch side, the backward one on st2 when given (the two
+// directions are independent within a phase).  *nlaunch: kernels launched.
 pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int maxP, int* nlaunch,
                           bool* handled, cudaStream_t st, cudaStream_t st2) {
     (void)maxP;
@@ -2079,15 +2063,12 @@ pgm_status launch_pm_tile(const LvlBatch& B, const MatchConst& mc, int nch, int 
         return launch_pm_direct(B, mc, nch, st);
     }
     const bool bits = use_bits(mc);
-    if (S[2].total <= both_limit(mc) && 2 * B.n <= PR_MAPS) {
+    if (one_launch(B, mc, S[2])) {
         const int words = G[0].words > G[1].words ? G[0].words : G[1].words;
         *nlaunch = 1;
         RowMaps& TM = pr_maps(B, nch, bits, S[2], G);
-        if (bits)
-            return nch == 2 ? launch_r<2, 0, 0, true>(B, mc, S[2], TM, words, st)
-                            : launch_r<6, 0, 0, true>(B, mc, S[2], TM, words, st);
-        return nch == 2 ? launch_both<2>(B, mc, S[2], G, TM, words, st)
-                        : launch_both<6>(B, mc, S[2], G, TM, words, st);
+        return nch == 2 ? launch_r<2, 0, 0, true>(B, mc, S[2], TM, words, st)
+                        : launch_r<6, 0, 0, true>(B, mc, S[2], TM, words, st);
     }
     for (int d = 0; d < 2; ++d) {
         if (S[d].total == 0) continue;
