@@ -154,6 +154,7 @@ def run_reference(a):
 # ------------------------------------------------------- ncu traffic record
 TRAFFIC_REC = os.path.join(ROOT, "profiles", "k_pm_r_traffic.json")
 PM_SRC = os.path.join(ROOT, "paper_1704_03217_gb300", "csrc", "pm_row.cu")
+PM_DIRECT_SRC = os.path.join(ROOT, "paper_1704_03217_gb300", "csrc", "pm_direct.cu")
 DEVICE_MARK = "// Host side: launch configuration.  No device code below this line.\n"
 # the capture the record is made from: DRAM counters of two level-0 search
 # launches (forward and backward of the second iteration's first colour phase)
@@ -171,7 +172,8 @@ def device_hash():
     text = open(PM_SRC, encoding="utf-8").read()
     if DEVICE_MARK not in text:
         return None
-    return hashlib.sha256(text.split(DEVICE_MARK)[0].encode("utf-8")).hexdigest()
+    text = text.split(DEVICE_MARK)[0] + open(PM_DIRECT_SRC, encoding="utf-8").read()
+    return hashlib.sha256(text.encode("utf-8")).hexdigest()
 
 
 def lattice_sizes(prm, w, h):
@@ -224,7 +226,8 @@ def write_traffic_record(csv_path):
                    "search launches per step (coarse levels assumed to move as many bytes per "
                    "seed as level 0, an upper bound: their data sit in L2)",
            "device_sha256": device_hash(),
-           "hash_note": "sha256 of pm_row.cu above the line " + json.dumps(DEVICE_MARK.strip())}
+           "hash_note": "sha256 of pm_row.cu above the line " + json.dumps(DEVICE_MARK.strip()) +
+                        " and of pm_direct.cu"}
     with open(TRAFFIC_REC, "w") as f:
         json.dump(rec, f, indent=1)
         f.write("\n")
@@ -705,7 +708,8 @@ def run_ours(a):
             "e2e": {"value": e2e, "unit": "pairs/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},
             "gpu_launches": int(launches),
-            "roofline": {"bound": "alu", "kernel": "k_pm_r (propagation + limited random search)",
+            "roofline": {"bound": "alu", "kernel": "k_pm_r, phases of few seeds k_pm_d "
+                                                 "(propagation + limited random search)",
                          "achieved": achieved_tmac, "peak": peak_tmac,
                          "unit": "Tmac/s (int16 x int16 element multiply-accumulates)",
                          "frac": achieved_tmac / peak_tmac, "traffic": traffic,
